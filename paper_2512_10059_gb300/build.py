@@ -6,6 +6,7 @@ Every ``csrc/*.cu`` file is compiled by nvcc in parallel (one ``-gencode``,
 A rebuild happens only when a source or header is newer than the library.
 """
 import glob
+import importlib.util
 import os
 import shutil
 import subprocess
@@ -18,7 +19,10 @@ OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libboys.so")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC,-fvisibility=hidden",
-         "--expt-relaxed-constexpr", "-I", CSRC, "-I", INCLUDE]
+         "--expt-relaxed-constexpr", "-I", CSRC, "-I", INCLUDE, "-I", OUT]
+# Tables that are generated at build time (too large to keep in the tree)
+LOCAL_GEN = os.path.join(CSRC, "gen_local.py")
+LOCAL_TABLES = os.path.join(OUT, "boys_local_tables.h")
 
 
 def nvcc() -> str:
@@ -34,7 +38,16 @@ def _sources():
 
 def _deps():
     return (_sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh"))
-            + glob.glob(os.path.join(INCLUDE, "*.h")) + [os.path.abspath(__file__)])
+            + glob.glob(os.path.join(INCLUDE, "*.h"))
+            + [LOCAL_GEN, os.path.join(CSRC, "gen_coeffs_fixed.py"), os.path.abspath(__file__)])
+
+
+def generate_tables():
+    spec = importlib.util.spec_from_file_location("gen_local", LOCAL_GEN)
+    gen = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(gen)
+    with open(LOCAL_TABLES, "w") as fh:
+        fh.write(gen.emit())
 
 
 def up_to_date() -> bool:
@@ -48,6 +61,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if not force and up_to_date():
         return LIB
     os.makedirs(OUT, exist_ok=True)
+    generate_tables()
     cc = nvcc()
     srcs = _sources()
 

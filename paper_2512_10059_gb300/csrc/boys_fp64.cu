@@ -1,35 +1,16 @@
-// FP64 stored mode (boys_eval) and fused consumer (boys_eval_fused).
+// FP64 stored mode (boys_eval, boys_eval_host) and fused consumer
+// (boys_eval_fused).
 //
-// Stored mode: one thread per argument (grid-stride loop, grid capped at 64
-// waves of resident blocks); KMAX is a template parameter so every loop is
-// unrolled.  A lane keeps only the first half of its orders: from the middle
-// step on every step completes two order-major rows for the whole warp, which
-// are written as full 256-byte segments (fp64::eval_store), and the register
-// count stays low enough for the occupancy that hides the integer-pipe
-// latency of the recurrence.
+// Stored mode: one thread per argument (grid-stride loop); KMAX is a template
+// parameter, the recurrence is unrolled, and each step writes one whole row of the
+// warp (256 bytes).
 #include <array>
 #include <utility>
 
 #include "boys_fp64.cuh"
 #include "boys_internal.h"
+#include "boys_region.cuh"
 
-// Minimum resident blocks per SM of the stored-mode kernel, which caps its
-// registers: swept on GB300 with the FP64-step table of boys_fp64.cuh
-// (N = 2^26, 8, 9, 10, 12 and 14 blocks at kmax 2, 4, 6, 8, 12, 16, 20, 24,
-// 28): up to kmax = 20 the 32-register cap of full occupancy is fastest
-// despite its spills to L1 (kmax 4: 1.86 ms against 1.91 with 8 and 1.90
-// with 12; kmax 12: 2.54 against 2.59 and 2.58; kmax 20: 3.33 against 3.39),
-// from kmax 24 on 8 blocks (64 registers) win (kmax 24: 3.79 against 4.22
-// with 14; kmax 32: 4.68 against 4.68 with 9 and 4.78 with 7).  Re-checked
-// with the 64-wave grid (8, 10, 12, 16 blocks): within 1% of the best at
-// every kmax.  BOYS_STORED_MIN_BLOCKS forces one value.
-constexpr int stored_min_blocks(int kmax) {
-#ifdef BOYS_STORED_MIN_BLOCKS
-    return BOYS_STORED_MIN_BLOCKS + 0 * kmax;
-#else
-    return kmax <= 20 ? 16 : 8;
-#endif
-}
 // FP64 recurrence steps and minimum resident blocks of the fused kernel.  Its
 // Horner sums add KMAX + 1 FMAs per argument to the FP64 pipe, so half of
 // stored mode's FP64 steps run in FP64.  Swept on GB300 at kmax 32, N = 2^26
@@ -53,12 +34,19 @@ namespace {
 
 constexpr int kBlock = 128;
 
-template <int KMAX, bool FULL_ROWS>
-__global__ void __launch_bounds__(kBlock, stored_min_blocks(KMAX)) k_eval_f64(const double* __restrict__ x, int64_t n,
+// Full occupancy (16 blocks of 128 threads per SM, 32 registers): the recurrence
+// keeps a dozen values, so the cap costs at most a few spills (kmax 8, 2^25
+// arguments: 478 us against 492 with 12 blocks and 492 with 10).
+// BOYS_STORED_MIN_BLOCKS forces another value.
+#ifndef BOYS_STORED_MIN_BLOCKS
+#define BOYS_STORED_MIN_BLOCKS 16
+#endif
+template <int KMAX>
+__global__ void __launch_bounds__(kBlock, BOYS_STORED_MIN_BLOCKS) k_eval_f64(const double* __restrict__ x, int64_t n,
                                                      double* __restrict__ out, int64_t ld) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-        fp64::eval_store<KMAX, FULL_ROWS>(__ldcs(x + i), out + i, ld);
+        region::eval_point<KMAX>(__ldcs(x + i), region::local_table<KMAX>(), region::Column::of<KMAX>(out + i, ld));
 }
 
 // |a|^E for a compile-time E >= 1, in the 64-bit-significand format (integer
@@ -140,10 +128,10 @@ __global__ void __launch_bounds__(kBlock, BOYS_FUSED_MIN_BLOCKS) k_fused_f64(con
     }
 }
 
-template <bool FULL_ROWS, int... K>
+template <int... K>
 constexpr auto eval_table(std::integer_sequence<int, K...>) {
     using Fn = void (*)(const double*, int64_t, double*, int64_t);
-    return std::array<Fn, sizeof...(K)>{&k_eval_f64<K, FULL_ROWS>...};
+    return std::array<Fn, sizeof...(K)>{&k_eval_f64<K>...};
 }
 
 template <int... K>
@@ -157,10 +145,9 @@ constexpr auto fused_table(std::integer_sequence<int, K...>) {
 
 
 namespace boys {
-// Checks and launches stored mode; full_rows selects the store pattern of
-// fp64::eval_store (true for output in host memory).
+// Checks and launches stored mode.
 static boys_status eval_launch(const char* name, const double* x, int64_t n, int kmax, double* out, int64_t ld,
-                               void* stream, bool full_rows) {
+                               void* stream) {
     if (kmax < 0 || kmax > 32) return fail(BOYS_ERR_KMAX, "%s: kmax=%d outside [0, 32]", name, kmax);
     if (n < 0) return fail(BOYS_ERR_INVALID_ARG, "%s: n=%lld < 0", name, (long long)n);
     if (ld < n) return fail(BOYS_ERR_INVALID_ARG, "%s: ld=%lld < n=%lld", name, (long long)ld, (long long)n);
@@ -168,11 +155,14 @@ static boys_status eval_launch(const char* name, const double* x, int64_t n, int
     if (!x || !out) return fail(BOYS_ERR_INVALID_ARG, "%s: NULL pointer", name);
     if (ld > INT64_MAX / (kmax + 1)) return fail(BOYS_ERR_INVALID_ARG, "%s: (kmax+1)*ld overflows", name);
     if (!aligned(x, 8) || !aligned(out, 8)) return fail(BOYS_ERR_ALIGNMENT, "%s: x/out not 8-byte aligned", name);
-    // one argument per thread, each order stored as soon as its row is complete
-    static constexpr auto tdev = eval_table<false>(std::make_integer_sequence<int, 33>{});
-    static constexpr auto thost = eval_table<true>(std::make_integer_sequence<int, 33>{});
-    const auto fn = full_rows ? thost[kmax] : tdev[kmax];
-    const int64_t grid = grid_for((const void*)fn, kBlock, n, (int64_t)kBlock);
+    static constexpr auto t = eval_table(std::make_integer_sequence<int, 33>{});
+    const auto fn = t[kmax];
+    // A block of a small order is over so soon that its launch shows: at most 8
+    // waves of resident blocks up to kmax 10 (kmax 0, 2^24 arguments: 83 us
+    // against 99 with 64 waves; kmax 8, 2^25: 478 against 483), the default 64
+    // above, where finer blocks balance the stores better (kmax 32, 2^26: 2.70 ms
+    // against 2.77 with 8).
+    const int64_t grid = grid_for((const void*)fn, kBlock, n, (int64_t)kBlock, kmax <= 10 ? 8 : BOYS_GRID_WAVES);
     fn<<<(unsigned)grid, kBlock, 0, (cudaStream_t)stream>>>(x, n, out, ld);
     return check_cuda(cudaGetLastError(), "boys_eval launch");
 }
@@ -180,7 +170,7 @@ static boys_status eval_launch(const char* name, const double* x, int64_t n, int
 
 BOYS_API boys_status boys_eval(const double* x, int64_t n, int kmax, double* out, int64_t ld,
                                void* stream) {
-    return boys::eval_launch("boys_eval", x, n, kmax, out, ld, stream, false);
+    return boys::eval_launch("boys_eval", x, n, kmax, out, ld, stream);
 }
 
 BOYS_API boys_status boys_eval_fused(const double* x, const double* rho, int64_t n, int kmax,
@@ -237,6 +227,5 @@ BOYS_API boys_status boys_eval_host(const double* x, int64_t n, int kmax, double
     if (st != BOYS_OK) return st;
     st = host_view(out, &od, "out");
     if (st != BOYS_OK) return st;
-    // full rows: partial writes over the host link are not merged
-    return eval_launch("boys_eval_host", (const double*)xd, n, kmax, (double*)od, ld, stream, true);
+    return eval_launch("boys_eval_host", (const double*)xd, n, kmax, (double*)od, ld, stream);
 }

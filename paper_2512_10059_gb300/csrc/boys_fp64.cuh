@@ -343,59 +343,5 @@ __device__ __forceinline__ void eval_point(double x, double (&F)[KMAX + 1]) {
     for (int k = 0; k <= KMAX; ++k) F[k] = S.inA ? v[KMAX - k] : v[k];
 }
 
-// Same values, stored by the whole warp: F_k(x) to col[k * ld].  Value number
-// p of the recurrence (p = 0 is the anchor) is F_{KMAX-p} on an A lane and
-// F_p on a B or C lane, so row k is complete once both p = k and p = KMAX-k
-// have been produced.  A lane therefore keeps its values p < KMAX/2 (at most
-// 17 doubles); from p >= KMAX/2 on, step p completes rows p and KMAX-p for
-// every lane of the warp and the two stores of that step cover both rows
-// completely between them, so L2 holds whole lines when they go to DRAM (a
-// value stored as soon as it is produced would leave rows partly written for
-// many steps, and L2 would evict partly written sectors that DRAM then
-// read-modify-writes).
-//
-// FULL_ROWS selects the store pattern.  false (device memory): each of the
-// step's two stores picks its row per lane, so each writes two half rows that
-// L2 merges before DRAM (cheaper on the ALU).  true (host memory over the
-// host link, where partial writes are not merged and would double the link
-// traffic): each store picks its value per lane and writes one full row.
-template <int KMAX, bool FULL_ROWS = false>
-__device__ __forceinline__ void eval_store(double x, double* __restrict__ col, int64_t ld) {
-    constexpr int H = KMAX / 2 + 1;
-    const Setup S = setup<KMAX, int_exp_for(KMAX, fp64_steps_for(KMAX))>(x);
-    double hold[H];
-    // Value p belongs to row KMAX - p on an A lane and to row p otherwise:
-    // row colp + p sld on every lane, and the held value's row colp + q sld
-    // (q = KMAX - p), with a lane's base and row stride chosen once.
-    double* const colp = S.inA ? col + (int64_t)KMAX * ld : col;
-    const int64_t sld = S.inA ? -ld : ld;
-    double yd = S.y0d;
-    xf::Xf y = S.y0;
-#pragma unroll
-    for (int p = 0; p <= KMAX; ++p) {
-        const double v = next_value<KMAX>(S, p, yd, y);
-        if (2 * p < KMAX) {
-            hold[p] = v;
-        } else if (2 * p == KMAX) {
-            __stcs(colp + p * sld, v);
-        } else {
-            // rows p and q = KMAX - p: this step's value is F_q on an A lane and
-            // F_p otherwise; the held one is the other.  Picking the row per
-            // lane (an address IMAD on the FMA pipe) instead of the value (two
-            // SELs per double on the ALU) makes each store write two half rows,
-            // which L2 merges before DRAM (kmax 32: 5.32 -> 5.24 ms; the lane's
-            // base and stride instead of a row select per store: 4.68 -> 4.65).
-            const int q = KMAX - p;
-            if (FULL_ROWS) {
-                __stcs(col + p * ld, S.inA ? hold[q] : v);
-                __stcs(col + q * ld, S.inA ? v : hold[q]);
-            } else {
-                __stcs(colp + p * sld, v);
-                __stcs(colp + q * sld, hold[q]);
-            }
-        }
-    }
-}
-
 }  // namespace fp64
 }  // namespace boys

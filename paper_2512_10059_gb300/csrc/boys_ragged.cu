@@ -26,8 +26,8 @@
 #include <utility>
 #include <vector>
 
-#include "boys_fp64.cuh"
 #include "boys_internal.h"
+#include "boys_region.cuh"
 
 namespace boys {
 namespace ragged {
@@ -48,11 +48,10 @@ struct Workspace {
 };
 static_assert(sizeof(Workspace) <= 256, "workspace fits its published size");
 
-// One argument's orders 0..K to dst[k * row]: the stored mode's evaluation
-// (same bits), which keeps only half of the orders live.
+// One argument's orders 0..K to dst[k * row]: the stored mode's evaluation (same bits).
 template <int K>
 __device__ __noinline__ void eval_store(double xv, double* __restrict__ dst, int64_t row) {
-    fp64::eval_store<K>(xv, dst, row);
+    region::eval_point<K>(xv, region::local_table<K>(), region::Column::of<K>(dst, row));
 }
 
 __device__ __forceinline__ void dispatch(int k, double xv, double* dst, int64_t row) {
@@ -209,7 +208,8 @@ __device__ __forceinline__ void group_tile(const double* __restrict__ x, const i
         const int64_t s0 = __ldg(seg_off + tl.seg);
         const int64_t row = __ldg(seg_off + tl.seg + 1) - s0;
         const int64_t j = tl.start + threadIdx.x;
-        fp64::eval_store<K>(__ldcs(x + s0 + j), out + __ldg(out_off + tl.seg) + j, row);
+        region::eval_point<K>(__ldcs(x + s0 + j), region::local_table<K>(),
+                              region::Column::of<K>(out + __ldg(out_off + tl.seg) + j, row));
     }
 }
 
