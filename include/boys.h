@@ -148,16 +148,17 @@ boys_status boys_grad(const double* x, int64_t n, int kmax, const double* g, int
  *                         * 256 bytes: one persistent launch over flat tiles,
  *                           taking tiles from a work counter in the workspace;
  *                         * boys_ragged_workspace_size_grouped(nseg, total)
- *                           bytes (more than 528 in general): the kmax-grouped
- *                           shape of a plan without a plan.  The call builds a
- *                           table of tiles (up to 128 arguments of one segment)
- *                           grouped by kmax in the workspace on the device,
- *                           then launches one kernel per kmax.  If the table
- *                           exceeds a smaller workspace (any size of at least
- *                           528 bytes selects this shape), those kernels do
- *                           nothing and a persistent launch runs instead.
+ *                           bytes: where they hold at least 40000 tiles (about
+ *                           5e6 arguments; smaller batches run as with 256
+ *                           bytes, which is faster), the tile shape of a plan
+ *                           without a plan.  The call builds a table of tiles
+ *                           (up to 128 arguments of one segment) sorted by
+ *                           kmax in the workspace on the device, then walks it
+ *                           with one launch.  If the table exceeds a smaller
+ *                           workspace, that launch does nothing and a
+ *                           persistent launch runs instead.
  *                       Either way everything is enqueued on `stream` with no
- *                       synchronisation (about 38 launches for the grouped shape).
+ *                       synchronisation.
  * Every argument is evaluated by the same code as boys_eval at its segment's
  * kmax, so results are bitwise identical to per-segment boys_eval calls, for
  * either shape.  Descriptors live on the device and are not validated on the
@@ -181,8 +182,8 @@ boys_status boys_ragged_status(const void* workspace, int* bad_kmax, void* strea
  * launch shape and captures it into a CUDA graph; boys_ragged_plan_launch then
  * replays it with one cudaGraphLaunch.  Shapes: the persistent kernel (block
  * size 64/128/256, 1 or 2 arguments per thread, 1 or 2 resident waves), or
- * waves = 0: one kernel per kmax present, each over a table of tiles of
- * `block` arguments built at creation, as parallel branches of the graph.
+ * waves = 0: one kernel over a table of tiles of `block` arguments, sorted by
+ * kmax, built at creation.
  * Every shape gives the same bits.  Creation reads the descriptors back (it
  * synchronises the device), validates them (seg_off[0] = 0, non-decreasing,
  * kmax in [0, 32]) and allocates a 256-byte workspace, and for waves = 0 the
@@ -195,7 +196,7 @@ boys_status boys_ragged_status(const void* workspace, int* bad_kmax, void* strea
  *                                   BOYS_AUTOTUNE_CACHE names a file, on disk.
  *   flags & BOYS_PLAN_FORCE_CONFIG  take the shape from BOYS_FORCE_CONFIG =
  *                                   "block,xpt,waves" (for tests; waves 0
- *                                   selects the per-kmax launches).
+ *                                   selects the tile table).
  * Without flags the default shape (128, 1, 1) is used.
  */
 #define BOYS_PLAN_AUTOTUNE 1

@@ -208,8 +208,8 @@ def boys_eval_ragged(x, seg_off, seg_kmax, out=None, out_off=None, workspace=Non
     """All segments of a ragged batch, without a plan.  Returns (out, out_off):
     segment s's F_k(x[seg_off[s]+j]) is at out[out_off[s] + k*len_s + j].
     Without ``workspace`` one of boys_ragged_workspace_size_grouped bytes is
-    allocated, which selects the kmax-grouped launches; a 256-byte workspace
-    selects the single persistent launch."""
+    allocated, which selects the kmax-grouped tiles for large batches; a 256-byte
+    workspace selects the single persistent launch."""
     x, seg_off, seg_kmax = _ragged_args(x, seg_off, seg_kmax)
     nseg = seg_kmax.numel()
     if out_off is None:
@@ -278,8 +278,8 @@ def ragged_status(workspace: torch.Tensor, stream=None) -> bool:
 
 class RaggedPlan:
     """A ragged batch bound to its buffers, with an autotuned launch shape and a
-    captured CUDA graph (workspace reset + persistent kernel, or one kernel per
-    kmax group as parallel branches: ``config()["waves"] == 0``).  ``launch()``
+    captured CUDA graph (workspace reset + persistent kernel, or one kernel over a
+    table of tiles sorted by kmax: ``config()["waves"] == 0``).  ``launch()``
     replays the graph on the current stream.  The tensors are kept alive by
     the plan."""
 

@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(kBlock, BOYS_STORED_MIN_BLOCKS) k_eval_f64(con
                                                      double* __restrict__ out, int64_t ld) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-        region::eval_point<KMAX>(__ldcs(x + i), region::local_table<KMAX>(), region::Column::of<KMAX>(out + i, ld));
+        region::eval_store<KMAX>(__ldcs(x + i), out + i, ld);
 }
 
 // |a|^E for a compile-time E >= 1, in the 64-bit-significand format (integer

@@ -31,15 +31,12 @@
 
 namespace boys {
 namespace ragged {
-
 constexpr int kMaxBlock = 256;
-// Resident blocks of kMaxBlock threads per SM the register allocation allows:
-// 4 caps the kernel at 64 registers.  The register count follows the largest
-// per-kmax body (kmax = 32, which then spills a little), and uncapped it held
-// the small-kmax bodies that dominate typical batches to a quarter of the
-// warps (2.40 ms vs 2.12 ms on 4096 segments at mean kmax 4.07).
+// Resident blocks of kMaxBlock threads per SM: 8 caps the kernels at 32 registers,
+// which every order's evaluation fits (4096 segments at mean kmax 4.07, 3.5e7
+// arguments: 560 us with 8, 612 with 6, 742 with 4).
 #ifndef BOYS_RAGGED_MIN_BLOCKS
-#define BOYS_RAGGED_MIN_BLOCKS 4
+#define BOYS_RAGGED_MIN_BLOCKS 8
 #endif
 
 struct Workspace {
@@ -51,7 +48,7 @@ static_assert(sizeof(Workspace) <= 256, "workspace fits its published size");
 // One argument's orders 0..K to dst[k * row]: the stored mode's evaluation (same bits).
 template <int K>
 __device__ __noinline__ void eval_store(double xv, double* __restrict__ dst, int64_t row) {
-    region::eval_point<K>(xv, region::local_table<K>(), region::Column::of<K>(dst, row));
+    region::eval_store<K>(xv, dst, row);
 }
 
 __device__ __forceinline__ void dispatch(int k, double xv, double* dst, int64_t row) {
@@ -174,14 +171,20 @@ __global__ void __launch_bounds__(kMaxBlock, BOYS_RAGGED_MIN_BLOCKS) k_ragged(co
     }
 }
 
-// ---------------------------------------------- kmax-grouped launches (plans)
+// ---------------------------------------------- kmax-grouped tiles
 //
-// A plan may instead launch one kernel per kmax present, each over a table of
-// tiles (up to blockDim consecutive arguments of one segment) built on the
-// host when the plan is created.  Every such kernel inlines one evaluation
-// body -- the stored mode's, so the bits are those of boys_eval -- with its
-// own register allocation, no segment search and no per-warp kmax dispatch;
-// the launches are parallel branches of the plan's graph.
+// The batch may instead be cut into tiles, each of up to blockDim consecutive
+// arguments of one segment, in a table sorted by the segments' kmax: built on the
+// host when a plan is created, or on the device at every plan-less call.  One
+// launch walks the table, largest kmax first.  A tile's kmax is the same for the
+// whole block, so the block takes one order's evaluation -- the stored mode's, same
+// bits -- with no segment search and no loop over the kmax of a warp.  All orders
+// fit in 32 registers, so one kernel holds them all at full occupancy.  One kernel
+// per kmax, as parallel graph branches of a plan or a chain of programmatic
+// dependents without one, ran large batches as fast (plan: 4096 segments, 3.5e7
+// arguments, 408 us either way) but paid for up to 33 launches (plan-less: 480 us
+// against 449; 512 segments, 4.3e5 arguments: plan 20 us against 11, plan-less 78
+// against 30).
 
 struct Tile {
     int32_t seg;    // segment index
@@ -190,16 +193,7 @@ struct Tile {
 };
 static_assert(sizeof(Tile) == 16, "tile table entries are 16 bytes");
 
-// 48 / 64 registers at 256 threads; BOYS_GROUPED_MIN_BLOCKS forces one value
-constexpr int grouped_min_blocks(int kmax) {
-#ifdef BOYS_GROUPED_MIN_BLOCKS
-    return BOYS_GROUPED_MIN_BLOCKS + 0 * kmax;
-#else
-    return kmax <= 16 ? 5 : 4;
-#endif
-}
-
-// One tile of a kmax group: its arguments, one per thread.
+// One tile: its arguments, one per thread.
 template <int K>
 __device__ __forceinline__ void group_tile(const double* __restrict__ x, const int64_t* __restrict__ seg_off,
                                            double* __restrict__ out, const int64_t* __restrict__ out_off,
@@ -208,40 +202,15 @@ __device__ __forceinline__ void group_tile(const double* __restrict__ x, const i
         const int64_t s0 = __ldg(seg_off + tl.seg);
         const int64_t row = __ldg(seg_off + tl.seg + 1) - s0;
         const int64_t j = tl.start + threadIdx.x;
-        region::eval_point<K>(__ldcs(x + s0 + j), region::local_table<K>(),
-                              region::Column::of<K>(out + __ldg(out_off + tl.seg) + j, row));
+        region::eval_store<K>(__ldcs(x + s0 + j), out + __ldg(out_off + tl.seg) + j, row);
     }
 }
 
-template <int K>
-__global__ void __launch_bounds__(kMaxBlock, grouped_min_blocks(K)) k_ragged_group(
-        const double* __restrict__ x, const int64_t* __restrict__ seg_off, double* __restrict__ out,
-        const int64_t* __restrict__ out_off, const Tile* __restrict__ tiles, int64_t ntiles) {
-    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) group_tile<K>(x, seg_off, out, out_off, tiles[t]);
-}
-
-using GroupFn = void (*)(const double*, const int64_t*, double*, const int64_t*, const Tile*, int64_t);
-
-template <int... K>
-constexpr auto group_table(std::integer_sequence<int, K...>) {
-    return std::array<GroupFn, sizeof...(K)>{&k_ragged_group<K>...};
-}
-
-// ------------------------------------ kmax-grouped launches without a plan
-//
-// With a large enough workspace, boys_eval_ragged builds the kmax-grouped tile
-// table itself, on the device, at every call: a count of tiles per kmax, an
-// exclusive scan of the 33 counts, and a fill in which each segment takes a
-// contiguous range of its group with one atomic (the order of tiles inside a
-// group varies, the values do not).  Then one kernel per kmax reads its
-// group's range from the workspace.  If the table would exceed the
-// workspace's capacity, the group kernels return at once and a persistent
-// launch, gated on that condition, evaluates the batch instead.
-
-constexpr int kGroupTile = 128;  // arguments per tile = threads per block of the group kernels
+constexpr int kGroupTile = 128;          // arguments per tile of a table built on the device
+constexpr size_t kMinTableTiles = 40000;  // smallest table that boys_eval_ragged builds
 
 struct GroupHeader {
-    Workspace ws;             // error word (the persistent fallback also uses next_tile)
+    Workspace ws;             // error word (the persistent kernel also uses next_tile)
     unsigned count[33];       // tiles per kmax
     unsigned base[33];        // first tile of each group
     unsigned cursor[33];      // fill positions
@@ -250,6 +219,42 @@ struct GroupHeader {
 };
 constexpr size_t kGroupHeaderBytes = 512;
 static_assert(sizeof(GroupHeader) <= kGroupHeaderBytes, "group header fits its reserved bytes");
+
+__global__ void __launch_bounds__(kMaxBlock, BOYS_RAGGED_MIN_BLOCKS) k_group(
+        const double* __restrict__ x, const int64_t* __restrict__ seg_off, double* __restrict__ out,
+        const int64_t* __restrict__ out_off, const Tile* __restrict__ tiles, const GroupHeader* __restrict__ h) {
+    if (h->overflow) return;
+    const unsigned total = h->total, lane = threadIdx.x & 31;
+    const unsigned base = h->base[lane + 1];  // first tile of kmax lane + 1
+    for (unsigned i = blockIdx.x; i < total; i += gridDim.x) {
+        const unsigned t = total - 1 - i;
+        const int k = __popc(__ballot_sync(0xffffffffu, base <= t));
+        const Tile tl = tiles[t];
+#define BOYS_GROUP_CASE(K) \
+    case K: group_tile<K>(x, seg_off, out, out_off, tl); break;
+        switch (k) {
+            BOYS_GROUP_CASE(0) BOYS_GROUP_CASE(1) BOYS_GROUP_CASE(2) BOYS_GROUP_CASE(3)
+            BOYS_GROUP_CASE(4) BOYS_GROUP_CASE(5) BOYS_GROUP_CASE(6) BOYS_GROUP_CASE(7)
+            BOYS_GROUP_CASE(8) BOYS_GROUP_CASE(9) BOYS_GROUP_CASE(10) BOYS_GROUP_CASE(11)
+            BOYS_GROUP_CASE(12) BOYS_GROUP_CASE(13) BOYS_GROUP_CASE(14) BOYS_GROUP_CASE(15)
+            BOYS_GROUP_CASE(16) BOYS_GROUP_CASE(17) BOYS_GROUP_CASE(18) BOYS_GROUP_CASE(19)
+            BOYS_GROUP_CASE(20) BOYS_GROUP_CASE(21) BOYS_GROUP_CASE(22) BOYS_GROUP_CASE(23)
+            BOYS_GROUP_CASE(24) BOYS_GROUP_CASE(25) BOYS_GROUP_CASE(26) BOYS_GROUP_CASE(27)
+            BOYS_GROUP_CASE(28) BOYS_GROUP_CASE(29) BOYS_GROUP_CASE(30) BOYS_GROUP_CASE(31)
+            BOYS_GROUP_CASE(32)
+        }
+#undef BOYS_GROUP_CASE
+    }
+}
+
+// ------------------------------------ kmax-grouped tiles without a plan
+//
+// With a large enough workspace, boys_eval_ragged builds the table itself, on the
+// device: a count of tiles per kmax, an exclusive scan of the 33 counts, and a fill
+// in which each segment takes a contiguous range of its group with one atomic
+// (the order of tiles inside a group varies, the values do not).  If the table
+// would exceed the workspace's capacity, the tile kernel returns at once and a
+// persistent launch, gated on that condition, evaluates the batch instead.
 
 __device__ __forceinline__ bool bad_kmax(int k) { return k < 0 || k > 32; }
 
@@ -295,27 +300,6 @@ __global__ void k_group_fill(const int64_t* __restrict__ seg_off, const int32_t*
     }
 }
 
-template <int K>
-__global__ void __launch_bounds__(kGroupTile, 2 * grouped_min_blocks(K)) k_ragged_group_dev(
-        const double* __restrict__ x, const int64_t* __restrict__ seg_off, double* __restrict__ out,
-        const int64_t* __restrict__ out_off, const Tile* __restrict__ tiles, const GroupHeader* __restrict__ h) {
-    // The groups write disjoint outputs and read only the finished table, so
-    // the next kmax's kernel may start at once (programmatic dependent launch):
-    // its blocks take the SMs as this kernel's blocks retire, with no drain.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (h->overflow) return;
-    const unsigned n = h->count[K];
-    const Tile* __restrict__ g = tiles + h->base[K];
-    for (unsigned t = blockIdx.x; t < n; t += gridDim.x) group_tile<K>(x, seg_off, out, out_off, g[t]);
-}
-
-using GroupDevFn = void (*)(const double*, const int64_t*, double*, const int64_t*, const Tile*, const GroupHeader*);
-
-template <int... K>
-constexpr auto group_dev_table(std::integer_sequence<int, K...>) {
-    return std::array<GroupDevFn, sizeof...(K)>{&k_ragged_group_dev<K>...};
-}
-
 using KernelFn = void (*)(const double*, const int64_t*, const int32_t*, int, double*, const int64_t*, Workspace*,
                           const unsigned*);
 
@@ -325,7 +309,7 @@ struct Config {
     int block = 128;
     int xpt = 1;
     int waves = 1;  // resident CTAs per SM multiplier for the persistent grid;
-                    // 0: one launch per kmax group (plans only; tile = block)
+                    // 0: kmax-grouped tiles (plans only; tile = block)
 };
 
 inline int grid_size(const Config& c) {
@@ -351,9 +335,17 @@ boys_status launch(const Config& c, const double* x, const int64_t* seg_off, con
     return check_cuda(cudaGetLastError(), "ragged launch");
 }
 
+// Blocks of the tile kernel for `tiles` tiles of `block` arguments: at most 16
+// waves of resident ones, so that the block scheduler evens out tiles of different
+// cost (4096 segments, 3.5e7 arguments: 408 us with 16 waves, 440 with 4, 467 with
+// 1, 416 with 64).
+inline unsigned group_grid(int64_t tiles, int block) {
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)sm_count() * (2048 / block) * 16));
+}
+
 // The plan-less kmax-grouped batch on a workspace of `bytes` >= kGroupHeaderBytes
-// + 16: reset the header, build the table on the device, one launch per kmax,
-// then the persistent kernel gated on the table's overflow flag.
+// + 16: reset the header, build the table on the device, walk it, then the
+// persistent kernel gated on the table's overflow flag.
 boys_status launch_grouped(const double* x, const int64_t* seg_off, const int32_t* seg_kmax, int32_t nseg, double* out,
                            const int64_t* out_off, void* workspace, size_t bytes, cudaStream_t stream) {
     GroupHeader* h = (GroupHeader*)workspace;
@@ -367,31 +359,10 @@ boys_status launch_grouped(const double* x, const int64_t* seg_off, const int32_
     k_group_scan<<<1, 32, 0, stream>>>(h, capacity);
     k_group_fill<<<sgrid, 256, 0, stream>>>(seg_off, seg_kmax, nseg, h, tiles);
     st = check_cuda(cudaGetLastError(), "ragged group table");
-    // One kernel per kmax, each launched as a programmatic dependent of the
-    // previous launch: a group kernel signals its dependents as it starts, and
-    // the fill kernel never does, so every group still starts after the table
-    // is complete.
-    static constexpr auto tg = group_dev_table(std::make_integer_sequence<int, 33>{});
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t lc = {};
-    lc.blockDim = dim3(kGroupTile);
-    lc.stream = stream;
-    lc.attrs = &attr;
-    lc.numAttrs = 1;
-    for (int k = 0; k <= 32 && st == BOYS_OK; ++k) {
-        lc.gridDim = dim3(sm_count() * blocks_per_sm((const void*)tg[k], kGroupTile));
-        st = check_cuda(cudaLaunchKernelEx(&lc, tg[k], x, seg_off, out, out_off, (const Tile*)tiles,
-                                           (const GroupHeader*)h), "ragged group launch");
-    }
-    if (st != BOYS_OK) return st;
+    k_group<<<group_grid((int64_t)capacity, kGroupTile), kGroupTile, 0, stream>>>(x, seg_off, out, out_off, tiles, h);
     const Config c;
-    lc.gridDim = dim3(grid_size(c));
-    lc.blockDim = dim3(c.block);
-    return check_cuda(cudaLaunchKernelEx(&lc, kernel_for(c.xpt), x, seg_off, seg_kmax, (int)nseg, out, out_off,
-                                         &h->ws, (const unsigned*)&h->overflow),
-                      "ragged fallback launch");
+    kernel_for(c.xpt)<<<grid_size(c), c.block, 0, stream>>>(x, seg_off, seg_kmax, nseg, out, out_off, &h->ws, &h->overflow);
+    return check_cuda(cudaGetLastError(), "ragged group launch");
 }
 
 // ------------------------------------------------------------- autotuning
@@ -487,12 +458,13 @@ struct boys_ragged_plan {
     cudaGraph_t graph;
     cudaGraphExec_t exec;
     float tuned_ms;
-    // kmax-grouped launches: host copies of the descriptors and the tile table
+    // kmax-grouped tiles: host copies of the descriptors, the tile table and its header
     std::vector<int64_t> off_host;
     std::vector<int32_t> km_host;
     ragged::Tile* tiles;
     int tiles_block;
-    int64_t group_begin[33], group_count[33];
+    ragged::GroupHeader* header;
+    int64_t ntiles;
 };
 
 BOYS_API size_t boys_ragged_workspace_size(void) { return 256; }
@@ -513,7 +485,11 @@ BOYS_API boys_status boys_eval_ragged(const double* x, const int64_t* seg_off, c
         return fail(BOYS_ERR_INVALID_ARG, "boys_eval_ragged: workspace_bytes=%zu < %zu", workspace_bytes,
                     boys_ragged_workspace_size());
     if (!aligned(workspace, 16)) return fail(BOYS_ERR_ALIGNMENT, "boys_eval_ragged: workspace not 16-byte aligned");
-    if (workspace_bytes >= ragged::kGroupHeaderBytes + sizeof(ragged::Tile))
+    // The table pays for itself (three kernels before the first tile) from about
+    // 40000 tiles on; smaller batches, whose workspace holds fewer, are left to the
+    // persistent kernel (5.2e6 arguments: 92 us either way; 4.3e5: 16 us against 30;
+    // 3.5e7: 560 against 449).
+    if (workspace_bytes >= ragged::kGroupHeaderBytes + ragged::kMinTableTiles * sizeof(ragged::Tile))
         return ragged::launch_grouped(x, seg_off, seg_kmax, nseg, out, out_off, workspace, workspace_bytes,
                                       (cudaStream_t)stream);
     ragged::Config c;
@@ -533,106 +509,64 @@ BOYS_API boys_status boys_ragged_status(const void* workspace, int* bad_kmax, vo
     return st;
 }
 
-// Tile table for tiles of `block` arguments: the tiles of every segment, grouped
-// by the segment's kmax (group k at [group_begin[k], + group_count[k])).
+// Tile table for tiles of `block` arguments, sorted by the segments' kmax, and
+// its header.
 static boys_status build_tiles(boys_ragged_plan* p, int block) {
-    if (p->tiles && p->tiles_block == block) return BOYS_OK;
+    if (p->tiles_block == block) return BOYS_OK;
     std::vector<ragged::Tile> tab;
+    ragged::GroupHeader h = {};
     for (int k = 0; k <= 32; ++k) {
-        p->group_begin[k] = (int64_t)tab.size();
+        h.base[k] = (unsigned)tab.size();
         for (int32_t sg = 0; sg < p->nseg; ++sg) {
             if (p->km_host[sg] != k) continue;
             const int64_t len = p->off_host[sg + 1] - p->off_host[sg];
             for (int64_t a = 0; a < len; a += block)
                 tab.push_back(ragged::Tile{sg, (int32_t)std::min<int64_t>(block, len - a), a});
         }
-        p->group_count[k] = (int64_t)tab.size() - p->group_begin[k];
+        h.count[k] = (unsigned)tab.size() - h.base[k];
     }
-    if (p->tiles) cudaFree(p->tiles);
+    if (tab.size() > 0xFFFFFFFFull) return fail(BOYS_ERR_INVALID_ARG, "boys_ragged_plan_create: too many tiles");
+    h.total = (unsigned)tab.size();
+    if (p->header) cudaFree(p->header);
+    p->header = nullptr;
     p->tiles = nullptr;
     p->tiles_block = 0;
-    if (tab.empty()) return BOYS_OK;
-    boys_status st = check_cuda(cudaMalloc((void**)&p->tiles, tab.size() * sizeof(ragged::Tile)), "plan tile table");
+    p->ntiles = (int64_t)tab.size();
+    const size_t bytes = ragged::kGroupHeaderBytes + std::max<size_t>(1, tab.size()) * sizeof(ragged::Tile);
+    boys_status st = check_cuda(cudaMalloc((void**)&p->header, bytes), "plan tile table");
     if (st != BOYS_OK) return st;
-    st = check_cuda(cudaMemcpy(p->tiles, tab.data(), tab.size() * sizeof(ragged::Tile), cudaMemcpyHostToDevice),
-                    "plan tile table upload");
+    p->tiles = (ragged::Tile*)((char*)p->header + ragged::kGroupHeaderBytes);
+    st = check_cuda(cudaMemcpy(p->header, &h, sizeof(h), cudaMemcpyHostToDevice), "plan tile table header");
+    if (st == BOYS_OK && !tab.empty())
+        st = check_cuda(cudaMemcpy(p->tiles, tab.data(), tab.size() * sizeof(ragged::Tile), cudaMemcpyHostToDevice),
+                        "plan tile table upload");
     if (st == BOYS_OK) p->tiles_block = block;
     return st;
 }
 
-// Streams and events that fork the kmax groups off the capturing stream and
-// join them back; created before the capture begins (object creation is not
-// a capturable operation) and destroyed after it ends.
-struct GroupFork {
-    cudaEvent_t fork = nullptr;
-    std::vector<int> ks;
-    std::vector<cudaStream_t> streams;
-    std::vector<cudaEvent_t> joins;
-    ~GroupFork() {
-        for (cudaEvent_t j : joins) cudaEventDestroy(j);
-        for (cudaStream_t g : streams) cudaStreamDestroy(g);
-        if (fork) cudaEventDestroy(fork);
-    }
-};
-
-static boys_status prepare_groups(boys_ragged_plan* p, const ragged::Config& c, GroupFork* f) {
-    boys_status st = build_tiles(p, c.block);  // allocates and copies: before any capture
-    if (st != BOYS_OK) return st;
-    st = check_cuda(cudaEventCreateWithFlags(&f->fork, cudaEventDisableTiming), "fork event");
-    for (int k = 0; k <= 32 && st == BOYS_OK; ++k) {
-        if (p->group_count[k] == 0) continue;
-        cudaStream_t g;
-        cudaEvent_t j;
-        st = check_cuda(cudaStreamCreateWithFlags(&g, cudaStreamNonBlocking), "group stream");
-        if (st != BOYS_OK) break;
-        f->streams.push_back(g);
-        st = check_cuda(cudaEventCreateWithFlags(&j, cudaEventDisableTiming), "join event");
-        if (st != BOYS_OK) break;
-        f->joins.push_back(j);
-        f->ks.push_back(k);
-    }
-    return st;
-}
-
 // Records the batch for configuration c on the capturing stream s: the
-// workspace reset, then either the persistent kernel or, for waves == 0, one
-// kernel per kmax group, forked onto their own streams and joined back.
-static boys_status record_launch(boys_ragged_plan* p, const ragged::Config& c, const GroupFork& f, cudaStream_t s) {
+// workspace reset, then the persistent kernel or, for waves == 0, the tile kernel.
+static boys_status record_launch(boys_ragged_plan* p, const ragged::Config& c, cudaStream_t s) {
     if (c.waves != 0)
         return ragged::launch(c, p->x, p->seg_off, p->seg_kmax, p->nseg, p->out, p->out_off, p->ws, s);
     boys_status st = check_cuda(cudaMemsetAsync(p->ws, 0, sizeof(ragged::Workspace), s), "ragged workspace reset");
     if (st != BOYS_OK) return st;
-    static constexpr auto tg = ragged::group_table(std::make_integer_sequence<int, 33>{});
-    st = check_cuda(cudaEventRecord(f.fork, s), "fork record");
-    for (size_t q = 0; q < f.ks.size() && st == BOYS_OK; ++q) {
-        const int k = f.ks[q];
-        const int64_t n = p->group_count[k];
-        int per_sm = 1;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tg[k], c.block, 0) != cudaSuccess || per_sm < 1)
-            per_sm = 1;
-        const int64_t grid = std::min<int64_t>(n, (int64_t)sm_count() * per_sm);
-        cudaStreamWaitEvent(f.streams[q], f.fork, 0);
-        tg[k]<<<(unsigned)grid, c.block, 0, f.streams[q]>>>(p->x, p->seg_off, p->out, p->out_off,
-                                                             p->tiles + p->group_begin[k], n);
-        st = check_cuda(cudaGetLastError(), "ragged group launch");
-        cudaEventRecord(f.joins[q], f.streams[q]);
-        cudaStreamWaitEvent(s, f.joins[q], 0);
-    }
-    return st;
+    ragged::k_group<<<ragged::group_grid(p->ntiles, c.block), c.block, 0, s>>>(p->x, p->seg_off, p->out, p->out_off,
+                                                                              p->tiles, p->header);
+    return check_cuda(cudaGetLastError(), "ragged group launch");
 }
 
 static boys_status capture(boys_ragged_plan* p, const ragged::Config& c, cudaGraph_t* graph, cudaGraphExec_t* exec) {
     *graph = nullptr;
     *exec = nullptr;
-    GroupFork f;
-    boys_status st = c.waves == 0 ? prepare_groups(p, c, &f) : BOYS_OK;
+    boys_status st = c.waves == 0 ? build_tiles(p, c.block) : BOYS_OK;  // allocates and copies: before any capture
     if (st != BOYS_OK) return st;
     cudaStream_t s;
     st = check_cuda(cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking), "plan stream");
     if (st != BOYS_OK) return st;
     st = check_cuda(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal), "begin capture");
     if (st == BOYS_OK) {
-        boys_status lst = record_launch(p, c, f, s);
+        boys_status lst = record_launch(p, c, s);
         cudaGraph_t g = nullptr;
         boys_status est = check_cuda(cudaStreamEndCapture(s, &g), "end capture");
         st = lst != BOYS_OK ? lst : est;
@@ -763,7 +697,7 @@ BOYS_API void boys_ragged_plan_destroy(boys_ragged_plan* plan) {
     if (plan->exec) cudaGraphExecDestroy(plan->exec);
     if (plan->graph) cudaGraphDestroy(plan->graph);
     if (plan->ws) cudaFree(plan->ws);
-    if (plan->tiles) cudaFree(plan->tiles);
+    if (plan->header) cudaFree(plan->header);
     delete plan;
 }
 

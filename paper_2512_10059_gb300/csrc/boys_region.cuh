@@ -108,7 +108,7 @@ __host__ __device__ constexpr u64 kappa(int l) {
     return ((top / d) << 32) + ((top % d) << 32) / d;
 }
 
-// T kappa_l / 2^64 for T < 0.56 2^64 (the recurrence's sums, see eval_point).
+// T kappa_l / 2^64 for T < 0.56 2^64 (the recurrence's sums, see eval_regular).
 template <int L>
 __device__ __forceinline__ u64 times_kappa(u64 T) {
     constexpr u64 k = kappa(L);
@@ -203,10 +203,18 @@ __device__ __forceinline__ double exponential(const State& S) {
     return S.Em == 0 ? 0.0 : e;
 }
 
-// Large, infinite and invalid arguments: rare, so a rolled loop, upward.  F_k
-// below the normal range flushes to zero, +inf gives 0, an invalid argument NaN.
+// x and -0.0 as 0; whether its bit pattern is one that start() takes, 0 <= x <= 2^28.
+__device__ __forceinline__ u64 bits_of(double x) {
+    const u64 xb = (u64)__double_as_longlong(x);
+    return (xb << 1) == 0 ? 0 : xb;
+}
+__device__ __forceinline__ bool regular(u64 xb) { return xb <= kBitsTwo28; }  // negative numbers and NaN lie above
+
+// Large, infinite and invalid arguments: rare, so a rolled loop, upward: to
+// out(k, value) with a run-time k.  F_k below the normal range flushes to zero, +inf
+// gives 0, an invalid argument NaN.
 template <int K, class Out>
-__device__ __noinline__ void eval_other(double x, Out& out) {
+__device__ __forceinline__ void eval_other(double x, Out&& out) {
     const long long xb = __double_as_longlong(x);
     const bool valid = xb >= 0 && xb <= fp64::kBitsInf;
     const xf::Xf r = xf::rsqrt(xf::from_double(!valid || xb > fp64::kBits1e300 ? 1e300 : x));
@@ -214,11 +222,10 @@ __device__ __noinline__ void eval_other(double x, Out& out) {
     const xf::Xf R = xf::mul(xf::Xf{r.m, r.e - 1}, r);
 #pragma unroll 1
     for (int j = 0; j <= K; ++j) {
-        out.template other<K>(j, valid ? xf::to_double(y) : fp64::quiet_nan());
+        out(j, valid ? xf::to_double(y) : fp64::quiet_nan());
         y = xf::mul_norm(xf::mul_raw(xf::odd(j), y), R);
     }
 }
-
 // Stores the orders of one argument: column `col` of rows `ld` apart.  The
 // address moves down a row at a time (addresses formed as col + k ld were all
 // kept in registers), with the carry flag (see mulhi; K = 16: 795 to 750 us for
@@ -238,8 +245,6 @@ struct Column {
             : "r"((unsigned)d), "r"((unsigned)(d >> 32)));
         row = (double*)((u64)hi << 32 | lo);
     }
-    template <int K>
-    __device__ __forceinline__ void other(int k, double v) const { row[(k - K) * ld] = v; }
 };
 
 // Recurrence steps in FP64, the first ones: two instructions and a ready value
@@ -250,23 +255,17 @@ struct Column {
 // cost what the steps save.
 constexpr int fp64_steps(int K) { return K < 6 ? 0 : K / 4; }
 
-// F_K, F_{K-1}, ..., F_0 at x, to out(integral_constant k, value); `tab` is the
-// order's table.  Arguments above 2^28, infinite and invalid ones go to
-// out.other<K>(k, value) instead, upward.
+// F_K, F_{K-1}, ..., F_LAST at a regular x, to out(integral_constant k, value);
+// `tab` is the order's table.
 //
 // A step, with u the scale of y: T = X y / 2^64 + (Em >> n) is (2l+1) F_l 2^(u-6), its
 // second term free in the product's accumulator, and y = T kappa_l / 2^64.  T stays
 // below 0.56 2^64 and above 2^56 (checked over A and B for every K by the integer
 // model of the tests; in C T < 2^63), so each value carries at least 53.9 correct bits
 // before it is cut to a double's.
-template <int K, int NF = fp64_steps(K), class Out>
-__device__ __forceinline__ void eval_point(double x, const Local* __restrict__ tab, Out&& out) {
-    u64 xb = (u64)__double_as_longlong(x);
-    if ((xb << 1) == 0) xb = 0;  // -0.0
-    if (xb > kBitsTwo28) {       // negative numbers and NaN too
-        eval_other<K>(x, out);
-        return;
-    }
+template <int K, int NF = fp64_steps(K), int LAST = 0, class Out>
+__device__ __forceinline__ void eval_regular(u64 xb, const Local* __restrict__ tab, Out&& out) {
+    const double x = __longlong_as_double((long long)xb);
     State S = start<K>(xb, tab);
     double yd = normalise<0>(S);
     out(std::integral_constant<int, K>{}, yd);
@@ -281,7 +280,7 @@ __device__ __forceinline__ void eval_point(double x, const Local* __restrict__ t
         S.y = ((yb & 0xFFFFFFFFFFFFFULL) | 0x10000000000000ULL) << 10;
         S.n = (int)(yb >> 52) - 1 - S.eb;
     }
-    unrolled<K - NF>([&](auto p) {
+    unrolled<K - NF - LAST>([&](auto p) {
         constexpr int l = K - 1 - NF - decltype(p)::value;
         const u64 T = mulhi(S.X, S.y, xf::shr_u64(S.Em, S.n));
         S.n += S.q;
@@ -294,6 +293,17 @@ __device__ __forceinline__ void eval_point(double x, const Local* __restrict__ t
             out(std::integral_constant<int, l>{}, normalise<gain>(S));
         }
     });
+}
+
+// All orders of one argument, to column `col` of rows `ld` apart.
+template <int K>
+__device__ __forceinline__ void eval_store(double x, double* col, int64_t ld) {
+    const u64 xb = bits_of(x);
+    if (regular(xb)) {
+        eval_regular<K>(xb, local_table<K>(), Column::of<K>(col, ld));
+    } else {
+        eval_other<K>(x, [col, ld](int k, double v) { col[k * ld] = v; });
+    }
 }
 
 }  // namespace region

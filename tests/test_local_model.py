@@ -1,4 +1,4 @@
-"""The FP64 evaluation of csrc/boys_region.cuh (start, eval_point), modelled with
+"""The FP64 evaluation of csrc/boys_region.cuh (start, eval_regular), modelled with
 Python integers operation by operation, on the tables that csrc/gen_local.py
 generates, against exact rational arithmetic on the printed coefficients: the
 anchors r_{A,k}, what the upward recurrence makes of r_B, and the asymptotic form,
