@@ -11,24 +11,6 @@
 #include "boys_internal.h"
 #include "boys_region.cuh"
 
-// FP64 recurrence steps and minimum resident blocks of the fused kernel.  Its
-// Horner sums add KMAX + 1 FMAs per argument to the FP64 pipe, so half of
-// stored mode's FP64 steps run in FP64.  Swept on GB300 at kmax 32, N = 2^26
-// (ms per launch): 8 blocks per SM with 6, 8, 10, 12 steps 6.65, 6.65, 6.79,
-// 7.19; 8 steps with 4, 5, 6, 7, 10, 12 blocks 6.50, 6.58, 6.50, 6.65, 6.78,
-// 6.75; 6 blocks with 6, 7, 9, 10 steps 6.56, 6.50, 6.57, 6.75.  The smaller
-// kmax follow the stored-mode table.  BOYS_FUSED_FP64_STEPS forces one value.
-constexpr int fused_fp64_steps(int kmax) {
-#ifdef BOYS_FUSED_FP64_STEPS
-    return BOYS_FUSED_FP64_STEPS + 0 * kmax;
-#else
-    return boys::fp64::fp64_steps_for(kmax) / 2;
-#endif
-}
-#ifndef BOYS_FUSED_MIN_BLOCKS
-#define BOYS_FUSED_MIN_BLOCKS 6
-#endif
-
 namespace boys {
 namespace {
 
@@ -49,82 +31,58 @@ __global__ void __launch_bounds__(kBlock, BOYS_STORED_MIN_BLOCKS) k_eval_f64(con
         region::eval_store<KMAX>(__ldcs(x + i), out + i, ld);
 }
 
-// |a|^E for a compile-time E >= 1, in the 64-bit-significand format (integer
-// pipes), by binary powering: about 2^-58 relative for E <= 17.
-template <int E>
-__device__ __forceinline__ xf::Xf xf_pow(xf::Xf b) {
-    xf::Xf r = b;
-    bool have = false;
-#pragma unroll
-    for (int bit = 0; (E >> bit) != 0; ++bit) {
-        if ((E >> bit) & 1) {
-            r = have ? xf::mul(r, b) : b;
-            have = true;
-        }
-        if ((E >> (bit + 1)) != 0) b = xf::mul(b, b);
+// The fused consumer is bound by the FP64 pipe: kmax FMAs an argument at 2 a clock
+// and SM (kmax 32, 2^24 arguments: 0.85 ms of the FMAs alone), so every step of the
+// recurrence stays on the integer pipes, and 8 blocks per SM suffice (8, 10, 12, 16
+// blocks: 990, 994, 1000, 994 us with 34 FP64 instructions an argument).
+#ifndef BOYS_FUSED_MIN_BLOCKS
+#define BOYS_FUSED_MIN_BLOCKS 8
+#endif
+
+// Horner sum in a, the orders as they come, from the highest down (order K first).
+template <int K>
+struct Horner {
+    double a, s;
+    template <int L>
+    __device__ __forceinline__ void operator()(std::integral_constant<int, L>, double v) {
+        s = L == K ? v : fma(s, a, v);
     }
-    return r;
+};
+
+// -2 v without the FP64 pipe where that is an exponent's increment.
+__device__ __forceinline__ double minus_twice(double v) {
+    const unsigned hi = (unsigned)__double2hiint(v), e = (hi >> 20) & 0x7FF;
+    if (e - 1 < 0x7FD) return __hiloint2double((int)((hi ^ 0x80000000u) + 0x100000u), __double2loint(v));
+    return -2.0 * v;  // zero, subnormal, 2^1023 and above, NaN
 }
 
-// out[i] = sum_k a^k F_k(x_i), a = -2 rho_i, as two Horner sums in a that
-// follow the order in which the step loop completes the orders.  Step p
-// yields value p of the recurrence, F_{KMAX-p} on an A lane and F_p on a B or
-// C lane; as in stored mode, a lane holds its values p < KMAX/2, and each
-// later step p completes the pair F_q, F_p (q = KMAX - p) on every lane.
-//   low  = sum_{k <= KH} a^k F_k, KH = KMAX/2: the F_q arrive with q
-//          descending, so the Horner sum runs as they come;
-//   high = sum_{j < NH} a^j F_{KH+1+j}: the F_p arrive ascending, so each
-//          lane parks them in its own shared-memory column and sums them
-//          afterwards;
-//   out  = low + a^(KH+1) high, the power on the integer pipes.
-// The lane never keeps all kmax+1 values, so nothing spills; the FP64 work is
-// the KMAX FMAs of a single Horner sum plus one.
+// The same for the arguments that eval_other takes, whose orders come upward.
+template <int KMAX>
+__device__ __noinline__ double fused_other(double x, double a) {
+    double f[KMAX + 1];
+    region::eval_other<KMAX>(x, [&](int k, double v) { f[k] = v; });
+    double s = f[KMAX];
+#pragma unroll 1
+    for (int k = KMAX - 1; k >= 0; --k) s = fma(s, a, f[k]);
+    return s;
+}
+
+// out[i] = sum_k a^k F_k(x_i), a = -2 rho_i.
 template <int KMAX>
 __global__ void __launch_bounds__(kBlock, BOYS_FUSED_MIN_BLOCKS) k_fused_f64(const double* __restrict__ x,
                                                       const double* __restrict__ rho, int64_t n,
                                                       double* __restrict__ out) {
-    constexpr int KH = KMAX / 2;
-    constexpr int NH = KMAX - KH;
-    constexpr int NF = fused_fp64_steps(KMAX);
-    __shared__ double s_high[NH > 0 ? NH : 1][kBlock];
-    double* const park = &s_high[0][threadIdx.x];
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        const fp64::Setup S = fp64::setup<KMAX, fp64::int_exp_for(KMAX, NF)>(__ldcs(x + i));
-        const double a = -2.0 * __ldcs(rho + i);
-        double hold[KH + 1];
-        double yd = S.y0d, low = 0.0;
-        xf::Xf y = S.y0;
-#pragma unroll
-        for (int p = 0; p <= KMAX; ++p) {
-            const double v = fp64::next_value<KMAX, NF>(S, p, yd, y);
-            if (2 * p < KMAX) {
-                hold[p] = v;
-            } else if (2 * p == KMAX) {
-                low = v;                                    // F_KH on every lane
-            } else {
-                const int q = KMAX - p;
-                const double fq = S.inA ? v : hold[q];
-                low = (q == KH) ? fq : fma(low, a, fq);     // q == KH: the first low term (odd KMAX)
-                park[(p - KH - 1) * kBlock] = S.inA ? hold[q] : v;  // F_p
-            }
+        const double xi = __ldcs(x + i), a = minus_twice(__ldcs(rho + i));
+        const region::u64 xb = region::bits_of(xi);
+        Horner<KMAX> h{a, 0.0};
+        if (region::regular(xb)) {
+            region::eval_regular<KMAX, 0>(xb, region::local_table<KMAX>(), h);
+        } else {
+            h.s = fused_other<KMAX>(xi, a);
         }
-        double r = low;
-        if (NH > 0) {
-            double high = park[(NH - 1) * kBlock];
-#pragma unroll
-            for (int j = NH - 2; j >= 0; --j) high = fma(high, a, park[j * kBlock]);
-            // a^(KH+1) from |a| on the integer pipes, with the sign of a^(KH+1);
-            // 0 for a zero or subnormal a (the format's zero must not be
-            // powered: its exponent would overflow)
-            const long long ab = __double_as_longlong(a);
-            const xf::Xf P = xf_pow<KH + 1>(xf::from_double(__longlong_as_double(ab & 0x7FFFFFFFFFFFFFFFLL)));
-            double w = P.e > 1023 ? __longlong_as_double(0x7FF0000000000000LL) : xf::to_double(P);
-            if ((ab & 0x7FF0000000000000LL) == 0) w = 0.0;
-            if (ab < 0 && ((KH + 1) & 1)) w = -w;
-            r = fma(w, high, low);
-        }
-        __stcs(out + i, r);
+        __stcs(out + i, h.s);
     }
 }
 

@@ -3,43 +3,58 @@
 // Differentiating the definition (Eq. 3) under the integral sign gives
 // dF_k/dx = -F_{k+1}, so for upstream gradients g_k:
 //     dL/dx_i = -sum_{k=0}^{kmax} g[k*ldg + i] * F_{k+1}(x_i).
-// The kernel re-evaluates F_0..F_{kmax+1} with the forward method at order
+// The kernel re-evaluates F_{kmax+1}..F_1 with the forward method at order
 // kmax+1 (nothing but x is saved by the forward), so kmax <= 31.
 #include <array>
 #include <utility>
 
-#include "boys_fp64.cuh"
 #include "boys_internal.h"
+#include "boys_region.cuh"
 
 namespace boys {
 namespace {
 
 constexpr int kBlock = 128;
 
-// FP64 recurrence steps and minimum resident blocks of the gradient kernel
-// (its own g_k F_{k+1} sum is FP64 work already): swept on GB300 at kmax 16,
-// N = 2^24: 4 FP64 steps and 8 blocks per SM (64 registers), 1.00 ms, against
-// 1.03 with 2, 1.02 with 6, 1.09 with 8 and, with an earlier step, 1.23 with
-// the register count left free.
-#ifndef BOYS_GRAD_FP64_STEPS
-#define BOYS_GRAD_FP64_STEPS 4
-#endif
+// The sum is kmax + 1 FMAs an argument on the FP64 pipe, at 2 a clock and SM (kmax
+// 16, 2^24 arguments: 0.45 ms of 0.56), so every step of the recurrence stays on
+// the integer pipes (958 us before, with the recurrence for all regions of
+// boys_fp64.cuh and 4 FP64 steps).  8 to 16 blocks per SM are within 1%.
 #ifndef BOYS_GRAD_MIN_BLOCKS
 #define BOYS_GRAD_MIN_BLOCKS 8
 #endif
+
+// Sums g_k F_{k+1} as the orders come, from the highest down.
+struct Dot {
+    const double* g;  // the next order's row
+    int64_t ldg;
+    double s;
+    template <int L>
+    __device__ __forceinline__ void operator()(std::integral_constant<int, L>, double v) {
+        s = fma(__ldcs(g), v, s);
+        g -= ldg;
+    }
+};
 
 template <int KMAX>
 __global__ void __launch_bounds__(kBlock, BOYS_GRAD_MIN_BLOCKS) k_grad_f64(const double* __restrict__ x, int64_t n,
                                                      const double* __restrict__ g, int64_t ldg,
                                                      double* __restrict__ dx) {
+    constexpr int K = KMAX + 1;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        double F[KMAX + 2];
-        fp64::eval_point<KMAX + 1, BOYS_GRAD_FP64_STEPS>(__ldcs(x + i), F);
-        double s = 0.0;
-#pragma unroll
-        for (int k = 0; k <= KMAX; ++k) s = fma(__ldcs(g + k * ldg + i), F[k + 1], s);
-        __stcs(dx + i, -s);
+        const double xi = __ldcs(x + i);
+        const region::u64 xb = region::bits_of(xi);
+        Dot d{g + KMAX * ldg + i, ldg, 0.0};
+        if (region::regular(xb)) {
+            region::eval_regular<K, 0, 1>(xb, region::local_table<K>(), d);
+        } else {
+            const double* gi = g + i;
+            region::eval_other<K>(xi, [&](int k, double v) {
+                if (k > 0) d.s = fma(__ldcs(gi + (k - 1) * ldg), v, d.s);
+            });
+        }
+        __stcs(dx + i, -d.s);
     }
 }
 
