@@ -61,8 +61,8 @@ HBM_FALLBACK_GBS = 6800.0
 # arguments it processes.  Valid only for the kernel sources it was taken on:
 # the bench reports traffic null whenever their SHA-256 differs.
 TRAFFIC_CAPTURE = {"bytes_per_x": 257.43, "sources_sha256": "573224284f6127327fe02ef0f56611de045fc7baafd59cb31ca99edbb94c00c2"}
-KERNEL_SOURCES = ("boys_fp64.cu", "boys_region.cuh", "gen_local.py", "boys_fp64.cuh", "boys_xf.cuh", "boys_math.cuh", "boys_coeffs_fp64.h",
-                  "boys_coeffs_fixed.h", "boys_xf_consts.h", "boys_exp_table.h", "boys_internal.h", "boys_abi.cu")
+KERNEL_SOURCES = ("boys_fp64.cu", "boys_region.cuh", "gen_local.py", "gen_coeffs_fixed.py", "boys_coeffs_fp64.h",
+                  "boys_xf.cuh", "boys_xf_consts.h", "boys_internal.h", "boys_abi.cu")
 
 
 def kernel_sources_sha256():

@@ -23,6 +23,7 @@ FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC,-fvisibility=hid
 # Tables that are generated at build time (too large to keep in the tree)
 LOCAL_GEN = os.path.join(CSRC, "gen_local.py")
 LOCAL_TABLES = os.path.join(OUT, "boys_local_tables.h")
+GRID_TABLE = os.path.join(OUT, "boys_grid_table.h")
 
 
 def nvcc() -> str:
@@ -46,8 +47,9 @@ def generate_tables():
     spec = importlib.util.spec_from_file_location("gen_local", LOCAL_GEN)
     gen = importlib.util.module_from_spec(spec)
     spec.loader.exec_module(gen)
-    with open(LOCAL_TABLES, "w") as fh:
-        fh.write(gen.emit())
+    for path, text in ((LOCAL_TABLES, gen.emit()), (GRID_TABLE, gen.emit_grid())):
+        with open(path, "w") as fh:
+            fh.write(text)
 
 
 def up_to_date() -> bool:

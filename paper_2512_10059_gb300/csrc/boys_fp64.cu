@@ -7,7 +7,6 @@
 #include <array>
 #include <utility>
 
-#include "boys_fp64.cuh"
 #include "boys_internal.h"
 #include "boys_region.cuh"
 

@@ -1,6 +1,6 @@
-// Double-precision elementary functions for the FP64 path, written for GB300's
-// FP64 budget (one DFMA costs the issue time of ~60 FFMAs, so every FP64
-// instruction saved is throughput).  Each is a published method, tested
+// Double-precision elementary functions written for GB300's FP64 budget (one DFMA
+// costs the issue time of ~60 FFMAs), offered by boys_diag_math; the evaluation
+// kernels take none of them.  Each is a published method, tested
 // against CUDA's own results in tests/test_math_fp64.py:
 //   * reciprocal / division: Newton–Raphson from the hardware seed
 //     (rcp.approx.ftz.f64, ~2^-20 relative), with the corrected quotient

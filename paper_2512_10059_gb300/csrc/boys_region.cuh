@@ -31,8 +31,9 @@
 #include <type_traits>
 #include <utility>
 
-#include "boys_fp64.cuh"
+#include "boys_coeffs_fp64.h"
 #include "boys_local_tables.h"
+#include "boys_xf.cuh"
 
 namespace boys {
 namespace region {
@@ -51,7 +52,13 @@ __device__ __forceinline__ void unrolled(F&& f) {
     unrolled(f, std::make_integer_sequence<int, N>{});
 }
 
+// Bit patterns: for non-negative doubles the IEEE order equals the integer order,
+// so the region tests run on the integer pipes.
+constexpr u64 kBitsX0 = BOYS_FP64_X0_BITS;
+constexpr u64 kBitsX1 = BOYS_FP64_X1_BITS;
 constexpr u64 kBitsTwo28 = 0x41B0000000000000ULL;
+constexpr long long kBitsInf = 0x7FF0000000000000LL;
+constexpr long long kBits1e300 = 0x7E37E43C8800759CLL;
 
 // One 64-byte entry of the expansion tables (gen_local.py).
 struct __align__(16) Local {
@@ -152,7 +159,7 @@ __device__ __forceinline__ double normalise(State& S) {
 template <int K>
 __device__ __forceinline__ State start(u64 xb, const Local* __restrict__ tab) {
     constexpr int kBitsC = K <= 12 ? 9 : 10;  // index bits of region C: one for the factor of two, log2 of its intervals
-    const bool inC = xb >= (u64)fp64::kBitsX1;
+    const bool inC = xb >= kBitsX1;
     const u64 m = (xb << 11) | 0x8000000000000000ULL;
     const int be = (int)(xb >> 52);
     State S;
@@ -165,7 +172,7 @@ __device__ __forceinline__ State start(u64 xb, const Local* __restrict__ tab) {
     const u64 v = (u64)vh << 32 | (unsigned)S.X;
     const int bits = inC ? kBitsC : 9;
     const int h = inC ? (be - 1023) >> 1 : 0;
-    const int first = inC ? BOYS_LOCAL_FIRST_C : xb >= (u64)fp64::kBitsX0 ? 1 : 0;
+    const int first = inC ? BOYS_LOCAL_FIRST_C : xb >= kBitsX0 ? 1 : 0;
     const Local* __restrict__ e = tab + (first + (int)(vh >> (32 - bits)));
     const u64 t = ~(v << bits);
     const unsigned t32 = (unsigned)(t >> 32);
@@ -216,13 +223,13 @@ __device__ __forceinline__ bool regular(u64 xb) { return xb <= kBitsTwo28; }  //
 template <int K, class Out>
 __device__ __forceinline__ void eval_other(double x, Out&& out) {
     const long long xb = __double_as_longlong(x);
-    const bool valid = xb >= 0 && xb <= fp64::kBitsInf;
-    const xf::Xf r = xf::rsqrt(xf::from_double(!valid || xb > fp64::kBits1e300 ? 1e300 : x));
-    xf::Xf y = xb == fp64::kBitsInf ? xf::zero() : xf::mul(xf::sqrt_pi_over_2(), r);
+    const bool valid = xb >= 0 && xb <= kBitsInf;
+    const xf::Xf r = xf::rsqrt(xf::from_double(!valid || xb > kBits1e300 ? 1e300 : x));
+    xf::Xf y = xb == kBitsInf ? xf::zero() : xf::mul(xf::sqrt_pi_over_2(), r);
     const xf::Xf R = xf::mul(xf::Xf{r.m, r.e - 1}, r);
 #pragma unroll 1
     for (int j = 0; j <= K; ++j) {
-        out(j, valid ? xf::to_double(y) : fp64::quiet_nan());
+        out(j, valid ? xf::to_double(y) : __longlong_as_double(0x7FF8000000000000LL));
         y = xf::mul_norm(xf::mul_raw(xf::odd(j), y), R);
     }
 }

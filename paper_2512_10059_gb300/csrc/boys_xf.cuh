@@ -2,28 +2,18 @@
 // integer pipes: value = m * 2^(e - 63) with 2^63 <= m < 2^64 (or m == 0 for
 // zero, whose exponent is kXfZeroExp so that it never dominates an addition).
 //
-// Why: on GB300 one FP64 instruction costs the issue time of ~60 FP32/INT
-// ones, and the Boys recurrences are 2 FP64 instructions per order.  Carried
-// out in this format they run on the integer pipes with about 2^-59 relative
-// rounding per operation (finer than FP64's 2^-53) and the full exponent
-// range, so the FP64 accuracy of the method (5e-14 absolute, Appendix B's
-// round-off analysis) is kept; results go back to IEEE doubles by integer
-// assembly of their bit patterns (truncation, < 1 ulp).
+// Why: on GB300 one FP64 instruction costs the issue time of ~60 FP32/INT ones.
+// In this format products and roots run on the integer pipes with about 2^-59
+// relative rounding per operation (finer than FP64's 2^-53) and the full exponent
+// range; results go back to IEEE doubles by integer assembly of their bit patterns
+// (truncation, < 1 ulp).  The evaluation itself (boys_region.cuh) uses it for the
+// arguments beyond its tables, the pairwise kernel for region C's closed form.
 //
-// The operations are built for the recurrence steps y' = (a y + s) c and cost
-// few instructions each:
 //  * products keep the high 64 bits of the 128-bit significand product from
 //    three 32 x 32-bit partial products (mulhi3: at most 2 units of 2^-64
 //    below the exact high half);
-//  * a sum aligns both terms to the larger exponent, one bit below the top,
-//    and is left unnormalised: the recurrences never cancel more than two
-//    leading bits (the upward step (2j+1) F_j - e^{-x} keeps at least 0.36
-//    of (2j+1) F_j on region B, and the downward step adds two positive
-//    terms), so a sum keeps its leading bit within its top four bits;
-//  * the product that follows a sum renormalises by a 32-bit leading-zero
-//    count of its high word, so a recurrence step renormalises once; the
-//    product feeding a sum skips renormalisation, and the addend e^{-x} is
-//    shifted and signed once per argument.
+//  * a raw product leaves its possible leading zero to the product that follows,
+//    which renormalises by a 32-bit leading-zero count of its high word.
 #pragma once
 
 #include <cstdint>
@@ -42,8 +32,6 @@ constexpr int kXfZeroExp = -(1 << 28);
 
 static __constant__ unsigned long long c_odd_m[64] = BOYS_XF_ODD_M_INIT;
 static __constant__ int c_odd_e[64] = BOYS_XF_ODD_E_INIT;
-static __constant__ unsigned long long c_rodd_m[64] = BOYS_XF_RECIP_ODD_M_INIT;
-static __constant__ int c_rodd_e[64] = BOYS_XF_RECIP_ODD_E_INIT;
 
 __device__ __forceinline__ Xf zero() { return Xf{0ULL, kXfZeroExp}; }
 
@@ -114,47 +102,15 @@ __device__ __forceinline__ Xf mul_raw(Xf a, Xf b) {
     return r;
 }
 
-// A signed addend prepared once: value = m * 2^(e - 62), |m| < 2^63.
-struct XfS {
-    long long m;
-    int e;
-};
-
-__device__ __forceinline__ XfS prepare_addend(Xf s, bool negate) {
-    const long long v = (long long)(s.m >> 1);
-    return XfS{negate ? -v : v, s.e};
-}
-
-// Logical and arithmetic right shifts by n >= 0 with PTX semantics: shift
-// counts of 64 and more give 0 (or the sign), so no clamp is needed.
+// Logical right shift by n >= 0 with PTX semantics: shift counts of 64 and more
+// give 0, so no clamp is needed.
 __device__ __forceinline__ unsigned long long shr_u64(unsigned long long a, int n) {
     unsigned long long r;
     asm("shr.b64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(n));
     return r;
 }
-__device__ __forceinline__ long long shr_s64(long long a, int n) {
-    long long r;
-    asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(n));
-    return r;
-}
-
-// t + s for a raw product t (m in [2^62, 2^64), or zero) and a prepared
-// signed addend s, where either both terms are >= 0 or the exact sum is at
-// least a quarter of t (the recurrences' cases).  Both terms are aligned to
-// 2^(E - 62), E the larger exponent (t one bit below the top, so two positive
-// terms cannot carry out), and added modulo 2^64.  The result is left
-// unnormalised for mul_norm: m = u with its leading bit in bits 59..63
-// (u >= t/4 >= 2^59 after the alignment), e = E + 1.  A zero sum stays zero
-// (m = 0, exponent near kXfZeroExp).
-__device__ __forceinline__ Xf add_raw(Xf t, XfS s) {
-    const int E = max(t.e, s.e);
-    const unsigned long long ta = shr_u64(t.m, E - t.e + 1);
-    const long long sa = shr_s64(s.m, E - s.e);  // arithmetic shift keeps the sign
-    return Xf{ta + (unsigned long long)sa, E + 1};
-}
-
-// a b for an operand a with at most four leading zeros (a sum from add_raw)
-// and a normalised b, renormalised by a 32-bit leading-zero count of the high
+// a b for an operand a with at most four leading zeros (a raw product) and a
+// normalised b, renormalised by a 32-bit leading-zero count of the high
 // word (the product's leading bit lies in bits 57..63; zero stays zero).
 // With the leading zeros of a the product keeps about 59 significant bits.
 __device__ __forceinline__ Xf mul_norm(Xf a, Xf b) {
@@ -253,9 +209,6 @@ __device__ __forceinline__ Xf exp_neg(double x) {
 }
 
 __device__ __forceinline__ Xf odd(int j) { return Xf{c_odd_m[j], c_odd_e[j]}; }        // 2j+1
-__device__ __forceinline__ Xf recip_odd(int l) { return Xf{c_rodd_m[l], c_rodd_e[l]}; }  // 1/(2l+1)
-
-__device__ __forceinline__ Xf select(bool p, Xf a, Xf b) { return p ? a : b; }
 
 }  // namespace xf
 }  // namespace boys

@@ -27,7 +27,10 @@ e^{-x} 2^(v-1) = w e / 2^64 with e = 2^63 e^{t/16}, and the exponents are
 n = v - 1 - u + 6 (low 16 bits) and 1079 - v (high 16 bits, signed).  In C, where
 e^{-x} counts as 0, w = 0 and the exponents are 1084 - u (for h = 0) and 0.
 
-Usage:  python gen_local.py > boys_local_tables.h
+A second table (``boys_grid_table.h``, for the pairwise kernel) holds F_m at the
+multiples of 1/16 up to 64 to the last bit of a double, m = 0..40.
+
+Usage:  python gen_local.py > boys_local_tables.h; python gen_local.py grid > boys_grid_table.h
 """
 import importlib.util
 import os
@@ -195,6 +198,38 @@ def table():
     return [ab + c for ab, c in zip(out, table_c())]
 
 
+GRID, GRID_ORDERS = 1024, 41
+
+
+def grid():
+    """F_m(j/16), m = 0..40, j = 1..1024, [m][j-1], scaled by 2^W, from the definition:
+    e^{-x} sum_i (2x)^i / ((2m+1)(2m+3)...(2m+2i+1)) at the highest order, downward below."""
+    edges, out = exp_neg_edges(GRID + 1), [[] for _ in range(GRID_ORDERS)]
+    for j in range(1, GRID + 1):
+        x2, m = (2 * j << W) // STEP, GRID_ORDERS - 1
+        term = total = (1 << W) // (2 * m + 1)
+        i = 0
+        while term:
+            i += 1
+            term = ((term * x2) >> W) // (2 * m + 2 * i + 1)
+            total += term
+        f = (total * edges[j]) >> W
+        out[m].append(f)
+        for m in range(GRID_ORDERS - 2, -1, -1):
+            f = (((f * x2) >> W) + edges[j]) // (2 * m + 1)
+            out[m].append(f)
+    return out
+
+
+def emit_grid():
+    """``boys_grid_table.h``: the grid's values as correctly rounded doubles."""
+    out = ["// F_m(j/16) as doubles; generated by gen_local.py when the library is built.", "#pragma once",
+           f"#define BOYS_GRID {GRID}", f"#define BOYS_GRID_ORDERS {GRID_ORDERS}",
+           "static __device__ const double g_grid_f[BOYS_GRID_ORDERS][BOYS_GRID] = {"]
+    out += ["{" + ",".join((v / (1 << W)).hex() for v in row) + "}," for row in grid()]
+    return "\n".join(out + ["};"]) + "\n"
+
+
 def emit():
     rows = table()
     out = ["// Local expansions of the anchors; generated by gen_local.py when the library is built.", "#pragma once",
@@ -210,4 +245,4 @@ def emit():
 
 if __name__ == "__main__":
     import sys
-    sys.stdout.write(emit())
+    sys.stdout.write(emit_grid() if "grid" in sys.argv else emit())
