@@ -146,15 +146,14 @@ boys_status boys_grad(const double* x, int64_t n, int kmax, const double* g, int
  *                         * 256 bytes: one persistent launch over flat tiles,
  *                           taking tiles from a work counter in the workspace;
  *                         * boys_ragged_workspace_size_grouped(nseg, total)
- *                           bytes: where they hold at least 40000 tiles (about
- *                           5e6 arguments; smaller batches run as with 256
- *                           bytes, which is faster), the tile shape of a plan
- *                           without a plan.  The call builds a table of tiles
- *                           (up to 128 arguments of one segment) sorted by
- *                           kmax in the workspace on the device, then walks it
- *                           with one launch.  If the table exceeds a smaller
- *                           workspace, that launch does nothing and a
- *                           persistent launch runs instead.
+ *                           bytes (any size of at least 528 selects this
+ *                           shape): the tile shape of a plan without a plan.
+ *                           The call builds a table of tiles (up to 128
+ *                           arguments of one segment) sorted by kmax in the
+ *                           workspace on the device, then walks it with one
+ *                           launch.  If the table exceeds a smaller workspace,
+ *                           that launch does nothing and a persistent launch
+ *                           runs instead.
  *                       Either way everything is enqueued on `stream` with no
  *                       synchronisation.
  * Every argument is evaluated by the same code as boys_eval at its segment's

@@ -231,8 +231,8 @@ def boys_eval_ragged(x, seg_off, seg_kmax, out=None, out_off=None, workspace=Non
     """All segments of a ragged batch, without a plan.  Returns (out, out_off):
     segment s's F_k(x[seg_off[s]+j]) is at out[out_off[s] + k*len_s + j].
     Without ``workspace`` one of boys_ragged_workspace_size_grouped bytes is
-    allocated, which selects the kmax-grouped tiles for large batches; a 256-byte
-    workspace selects the single persistent launch."""
+    allocated, which selects the kmax-grouped tiles; a 256-byte workspace selects
+    the single persistent launch."""
     x, seg_off, seg_kmax = _ragged_args(x, seg_off, seg_kmax)
     nseg = seg_kmax.numel()
     if out_off is None:

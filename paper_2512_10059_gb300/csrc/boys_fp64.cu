@@ -59,7 +59,7 @@ __device__ __forceinline__ double minus_twice(double v) {
 template <int KMAX>
 __device__ __noinline__ double fused_other(double x, double a) {
     double f[KMAX + 1];
-    region::eval_other<KMAX>(x, [&](int k, double v) { f[k] = v; });
+    region::eval_other(KMAX, x, [&](int k, double v) { f[k] = v; });
     double s = f[KMAX];
 #pragma unroll 1
     for (int k = KMAX - 1; k >= 0; --k) s = fma(s, a, f[k]);

@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(kBlock, BOYS_GRAD_MIN_BLOCKS) k_grad_f64(const
             region::eval_regular<K, 0, 1>(xb, region::local_table<K>(), d);
         } else {
             const double* gi = g + i;
-            region::eval_other<K>(xi, [&](int k, double v) {
+            region::eval_other(K, xi, [&](int k, double v) {
                 if (k > 0) d.s = fma(__ldcs(gi + (k - 1) * ldg), v, d.s);
             });
         }

@@ -132,7 +132,7 @@ __device__ __noinline__ double w_direct(double X, const double* c, const long lo
     const u64 xb = region::bits_of(X);
     Weighted w{c, 0.0};
     if (!region::regular(xb)) {
-        region::eval_other<K>(X, [&](int k, double v) { w.s = fma(c[k], v, w.s); });
+        region::eval_other(K, X, [&](int k, double v) { w.s = fma(c[k], v, w.s); });
         return w.s;
     }
     if (xb < region::kBitsX1 || fe == kNotFinite) {

@@ -48,7 +48,7 @@ static_assert(sizeof(Workspace) <= 256, "workspace fits its published size");
 // One argument's orders 0..K to dst[k * row]: the stored mode's evaluation (same bits).
 template <int K>
 __device__ __noinline__ void eval_store(double xv, double* __restrict__ dst, int64_t row) {
-    region::eval_store<K>(xv, dst, row);
+    region::eval_store<K, true>(xv, dst, row);
 }
 
 __device__ __forceinline__ void dispatch(int k, double xv, double* dst, int64_t row) {
@@ -183,8 +183,9 @@ __global__ void __launch_bounds__(kMaxBlock, BOYS_RAGGED_MIN_BLOCKS) k_ragged(co
 // per kmax, as parallel graph branches of a plan or a chain of programmatic
 // dependents without one, ran large batches as fast (plan: 4096 segments, 3.5e7
 // arguments, 408 us either way) but paid for up to 33 launches (plan-less: 480 us
-// against 449; 512 segments, 4.3e5 arguments: plan 20 us against 11, plan-less 78
-// against 30).
+// against 422; 512 segments, 4.3e5 arguments: plan 20 us against 11, plan-less 78
+// against 16, as fast as the persistent kernel).  The loop for irregular arguments is
+// shared by the orders: a copy in each made the kernel's code larger (plan 432 us).
 
 struct Tile {
     int32_t seg;    // segment index
@@ -202,12 +203,11 @@ __device__ __forceinline__ void group_tile(const double* __restrict__ x, const i
         const int64_t s0 = __ldg(seg_off + tl.seg);
         const int64_t row = __ldg(seg_off + tl.seg + 1) - s0;
         const int64_t j = tl.start + threadIdx.x;
-        region::eval_store<K>(__ldcs(x + s0 + j), out + __ldg(out_off + tl.seg) + j, row);
+        region::eval_store<K, true>(__ldcs(x + s0 + j), out + __ldg(out_off + tl.seg) + j, row);
     }
 }
 
-constexpr int kGroupTile = 128;          // arguments per tile of a table built on the device
-constexpr size_t kMinTableTiles = 40000;  // smallest table that boys_eval_ragged builds
+constexpr int kGroupTile = 128;  // arguments per tile of a table built on the device
 
 struct GroupHeader {
     Workspace ws;             // error word (the persistent kernel also uses next_tile)
@@ -250,9 +250,10 @@ __global__ void __launch_bounds__(kMaxBlock, BOYS_RAGGED_MIN_BLOCKS) k_group(
 // ------------------------------------ kmax-grouped tiles without a plan
 //
 // With a large enough workspace, boys_eval_ragged builds the table itself, on the
-// device: a count of tiles per kmax, an exclusive scan of the 33 counts, and a fill
-// in which each segment takes a contiguous range of its group with one atomic
-// (the order of tiles inside a group varies, the values do not).  If the table
+// device: a count of tiles per kmax, an exclusive scan of the 33 counts (by one warp;
+// one thread after another took 10 us), and a fill in which each segment takes a
+// contiguous range of its group with one atomic and a warp writes it (the order of
+// tiles inside a group varies, the values do not).  If the table
 // would exceed the workspace's capacity, the tile kernel returns at once and a
 // persistent launch, gated on that condition, evaluates the batch instead.
 
@@ -272,30 +273,43 @@ __global__ void k_group_count(const int64_t* __restrict__ seg_off, const int32_t
     }
 }
 
+// One warp: lane k takes order k, and all of them order 32.
 __global__ void k_group_scan(GroupHeader* __restrict__ h, unsigned long long capacity) {
-    if (threadIdx.x != 0) return;
-    unsigned long long run = 0;
-    for (int k = 0; k <= 32; ++k) {
-        h->base[k] = (unsigned)run;
-        h->cursor[k] = (unsigned)run;
-        run += h->count[k];
+    const unsigned lane = threadIdx.x, mine = h->count[lane];
+    unsigned run = mine;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned u = __shfl_up_sync(0xffffffffu, run, d);
+        if (lane >= d) run += u;
     }
-    h->total = (unsigned)run;
-    h->overflow = run > capacity ? 1u : 0u;
+    h->base[lane] = run - mine;
+    h->cursor[lane] = run - mine;
+    if (lane == 31) {
+        const unsigned long long total = (unsigned long long)run + h->count[32];
+        h->base[32] = run;
+        h->cursor[32] = run;
+        h->total = (unsigned)total;
+        h->overflow = total > capacity ? 1u : 0u;
+    }
 }
 
+// A warp per segment: its tiles are written side by side.
 __global__ void k_group_fill(const int64_t* __restrict__ seg_off, const int32_t* __restrict__ seg_kmax, int nseg,
                              GroupHeader* __restrict__ h, Tile* __restrict__ tiles) {
     if (h->overflow) return;
-    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < nseg; s += gridDim.x * blockDim.x) {
+    const unsigned lane = threadIdx.x & 31;
+    const int64_t warps = (int64_t)gridDim.x * blockDim.x / 32;
+    for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32; s < nseg; s += warps) {
         const int64_t len = __ldg(seg_off + s + 1) - __ldg(seg_off + s);
         const int k = __ldg(seg_kmax + s);
         if (len <= 0 || bad_kmax(k)) continue;
         const unsigned n = (unsigned)((len + kGroupTile - 1) / kGroupTile);
-        const unsigned p = atomicAdd(&h->cursor[k], n);
-        for (unsigned t = 0; t < n; ++t) {
+        unsigned p = 0;
+        if (lane == 0) p = atomicAdd(&h->cursor[k], n);
+        p = __shfl_sync(0xffffffffu, p, 0);
+        for (unsigned t = lane; t < n; t += 32) {
             const int64_t a = (int64_t)t * kGroupTile;
-            tiles[p + t] = Tile{s, (int32_t)min((int64_t)kGroupTile, len - a), a};
+            tiles[p + t] = Tile{(int32_t)s, (int32_t)min((int64_t)kGroupTile, len - a), a};
         }
     }
 }
@@ -357,7 +371,8 @@ boys_status launch_grouped(const double* x, const int64_t* seg_off, const int32_
     const int sgrid = (int)std::min<int64_t>((nseg + 255) / 256, (int64_t)sm_count() * 4);
     k_group_count<<<sgrid, 256, 0, stream>>>(seg_off, seg_kmax, nseg, h);
     k_group_scan<<<1, 32, 0, stream>>>(h, capacity);
-    k_group_fill<<<sgrid, 256, 0, stream>>>(seg_off, seg_kmax, nseg, h, tiles);
+    const int fgrid = (int)std::min<int64_t>(((int64_t)nseg * 32 + 255) / 256, (int64_t)sm_count() * 8);
+    k_group_fill<<<fgrid, 256, 0, stream>>>(seg_off, seg_kmax, nseg, h, tiles);
     st = check_cuda(cudaGetLastError(), "ragged group table");
     k_group<<<group_grid((int64_t)capacity, kGroupTile), kGroupTile, 0, stream>>>(x, seg_off, out, out_off, tiles, h);
     const Config c;
@@ -485,11 +500,7 @@ BOYS_API boys_status boys_eval_ragged(const double* x, const int64_t* seg_off, c
         return fail(BOYS_ERR_INVALID_ARG, "boys_eval_ragged: workspace_bytes=%zu < %zu", workspace_bytes,
                     boys_ragged_workspace_size());
     if (!aligned(workspace, 16)) return fail(BOYS_ERR_ALIGNMENT, "boys_eval_ragged: workspace not 16-byte aligned");
-    // The table pays for itself (three kernels before the first tile) from about
-    // 40000 tiles on; smaller batches, whose workspace holds fewer, are left to the
-    // persistent kernel (5.2e6 arguments: 92 us either way; 4.3e5: 16 us against 30;
-    // 3.5e7: 560 against 449).
-    if (workspace_bytes >= ragged::kGroupHeaderBytes + ragged::kMinTableTiles * sizeof(ragged::Tile))
+    if (workspace_bytes >= ragged::kGroupHeaderBytes + sizeof(ragged::Tile))
         return ragged::launch_grouped(x, seg_off, seg_kmax, nseg, out, out_off, workspace, workspace_bytes,
                                       (cudaStream_t)stream);
     ragged::Config c;

@@ -220,8 +220,8 @@ __device__ __forceinline__ bool regular(u64 xb) { return xb <= kBitsTwo28; }  //
 // Large, infinite and invalid arguments: rare, so a rolled loop, upward: to
 // out(k, value) with a run-time k.  F_k below the normal range flushes to zero, +inf
 // gives 0, an invalid argument NaN.
-template <int K, class Out>
-__device__ __forceinline__ void eval_other(double x, Out&& out) {
+template <class Out>
+__device__ __forceinline__ void eval_other(int K, double x, Out&& out) {
     const long long xb = __double_as_longlong(x);
     const bool valid = xb >= 0 && xb <= kBitsInf;
     const xf::Xf r = xf::rsqrt(xf::from_double(!valid || xb > kBits1e300 ? 1e300 : x));
@@ -302,14 +302,21 @@ __device__ __forceinline__ void eval_regular(u64 xb, const Local* __restrict__ t
     });
 }
 
-// All orders of one argument, to column `col` of rows `ld` apart.
-template <int K>
+static __device__ __noinline__ void store_other(int K, double x, double* col, int64_t ld) {
+    eval_other(K, x, [col, ld](int k, double v) { col[k * ld] = v; });
+}
+
+// All orders of one argument, to column `col` of rows `ld` apart.  A kernel of many
+// orders keeps one copy of the loop for irregular arguments (kShared), out of line.
+template <int K, bool kShared = false>
 __device__ __forceinline__ void eval_store(double x, double* col, int64_t ld) {
     const u64 xb = bits_of(x);
     if (regular(xb)) {
         eval_regular<K>(xb, local_table<K>(), Column::of<K>(col, ld));
+    } else if (kShared) {
+        store_other(K, x, col, ld);
     } else {
-        eval_other<K>(x, [col, ld](int k, double v) { col[k * ld] = v; });
+        eval_other(K, x, [col, ld](int k, double v) { col[k * ld] = v; });
     }
 }
 

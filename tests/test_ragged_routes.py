@@ -1,7 +1,6 @@
-"""The three routes of boys_eval_ragged by the size of the workspace and of the
-batch: the persistent kernel (256 bytes, or room for fewer than 40000 tiles), the
-tile table built on the device, and the persistent kernel behind a table that
-does not fit.  All give the bits of flat boys_eval."""
+"""The three routes of boys_eval_ragged by the size of the workspace: the persistent
+kernel (256 bytes), the tile table built on the device, and the persistent kernel
+behind a table that does not fit.  All give the bits of flat boys_eval."""
 import numpy as np
 import pytest
 import torch
