@@ -31,9 +31,10 @@ __global__ void __launch_bounds__(kBlock, BOYS_STORED_MIN_BLOCKS) k_eval_f64(con
 }
 
 // The fused consumer is bound by the FP64 pipe: kmax FMAs an argument at 2 a clock
-// and SM (kmax 32, 2^24 arguments: 0.85 ms of the FMAs alone), so every step of the
-// recurrence stays on the integer pipes, and 8 blocks per SM suffice (8, 10, 12, 16
-// blocks: 990, 994, 1000, 994 us with 34 FP64 instructions an argument).
+// and SM (kmax 32, 2^24 arguments: 853 us of the 886), so every step of the recurrence
+// stays on the integer pipes, and so does everything else (with two more FP64
+// instructions an argument, the factor -2 and a comparison, 964 us).  8 blocks per SM
+// suffice (8, 10, 12, 16 blocks: within 1%).
 #ifndef BOYS_FUSED_MIN_BLOCKS
 #define BOYS_FUSED_MIN_BLOCKS 8
 #endif
@@ -48,11 +49,13 @@ struct Horner {
     }
 };
 
-// -2 v without the FP64 pipe where that is an exponent's increment.
+// -2 v without the FP64 pipe where that is an exponent's increment (the product in
+// the same function would be computed every time and selected).
+static __device__ __noinline__ double minus_twice_special(double v) { return -2.0 * v; }
 __device__ __forceinline__ double minus_twice(double v) {
     const unsigned hi = (unsigned)__double2hiint(v), e = (hi >> 20) & 0x7FF;
     if (e - 1 < 0x7FD) return __hiloint2double((int)((hi ^ 0x80000000u) + 0x100000u), __double2loint(v));
-    return -2.0 * v;  // zero, subnormal, 2^1023 and above, NaN
+    return minus_twice_special(v);  // zero, subnormal, 2^1023 and above, NaN
 }
 
 // The same for the arguments that eval_other takes, whose orders come upward.

@@ -17,21 +17,21 @@ namespace {
 constexpr int kBlock = 128;
 
 // The sum is kmax + 1 FMAs an argument on the FP64 pipe, at 2 a clock and SM (kmax
-// 16, 2^24 arguments: 0.45 ms of 0.56), so every step of the recurrence stays on
-// the integer pipes (958 us before, with the recurrence for all regions of
-// boys_fp64.cuh and 4 FP64 steps).  8 to 16 blocks per SM are within 1%.
+// 16, 2^24 arguments: 453 us of about 500; 561 with two more FP64 instructions, 958 with
+// the recurrence that served all regions), so every step of the recurrence stays on
+// the integer pipes.  8 to 16 blocks per SM are within 1%.
 #ifndef BOYS_GRAD_MIN_BLOCKS
 #define BOYS_GRAD_MIN_BLOCKS 8
 #endif
 
-// Sums g_k F_{k+1} as the orders come, from the highest down.
+// Subtracts g_k F_{k+1} as the orders come, from the highest down.
 struct Dot {
     const double* g;  // the next order's row
     int64_t ldg;
     double s;
     template <int L>
     __device__ __forceinline__ void operator()(std::integral_constant<int, L>, double v) {
-        s = fma(__ldcs(g), v, s);
+        s = fma(-__ldcs(g), v, s);
         g -= ldg;
     }
 };
@@ -51,10 +51,10 @@ __global__ void __launch_bounds__(kBlock, BOYS_GRAD_MIN_BLOCKS) k_grad_f64(const
         } else {
             const double* gi = g + i;
             region::eval_other(K, xi, [&](int k, double v) {
-                if (k > 0) d.s = fma(__ldcs(gi + (k - 1) * ldg), v, d.s);
+                if (k > 0) d.s = fma(-__ldcs(gi + (k - 1) * ldg), v, d.s);
             });
         }
-        __stcs(dx + i, -d.s);
+        __stcs(dx + i, d.s);
     }
 }
 

@@ -211,9 +211,11 @@ __device__ __forceinline__ double exponential(const State& S) {
 }
 
 // x and -0.0 as 0; whether its bit pattern is one that start() takes, 0 <= x <= 2^28.
+// (The test for -0.0 by halves: as one 64-bit comparison it becomes an FP64 one.)
 __device__ __forceinline__ u64 bits_of(double x) {
-    const u64 xb = (u64)__double_as_longlong(x);
-    return (xb << 1) == 0 ? 0 : xb;
+    const unsigned lo = (unsigned)__double2loint(x), hi = (unsigned)__double2hiint(x);
+    const unsigned h = (lo | (hi ^ 0x80000000u)) == 0 ? 0 : hi;
+    return (u64)h << 32 | lo;
 }
 __device__ __forceinline__ bool regular(u64 xb) { return xb <= kBitsTwo28; }  // negative numbers and NaN lie above
 
