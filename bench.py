@@ -60,7 +60,7 @@ HBM_FALLBACK_GBS = 6800.0
 # (profiles/k_eval_f64_kmax32_eri_mixture.md), scaled to the launch by the
 # arguments it processes.  Valid only for the kernel sources it was taken on:
 # the bench reports traffic null whenever their SHA-256 differs.
-TRAFFIC_CAPTURE = {"bytes_per_x": 257.43, "sources_sha256": "573224284f6127327fe02ef0f56611de045fc7baafd59cb31ca99edbb94c00c2"}
+TRAFFIC_CAPTURE = {"bytes_per_x": 257.67, "sources_sha256": "446793f29f1761891e7d8aa3ba8633d08572be981e2a0dc66b7805e0b4065baf"}
 KERNEL_SOURCES = ("boys_fp64.cu", "boys_region.cuh", "gen_local.py", "gen_coeffs_fixed.py", "boys_coeffs_fp64.h",
                   "boys_xf.cuh", "boys_xf_consts.h", "boys_internal.h", "boys_abi.cu")
 
@@ -331,9 +331,9 @@ def run_ours(args):
     flops_per_launch = n * fpx
     # Primary roof: HBM, the hard floor of stored mode (8 + 8*33 bytes per
     # argument must move).  The paper's algorithmic FP64 work per argument is
-    # reported beside it: the kernel runs much of it (e^{-x}, the anchors'
-    # inverse square root, most recurrence steps) on the integer pipes, so
-    # that fraction can exceed 1 and does not bound the kernel.
+    # reported beside it: the kernel runs most of it on the integer pipes (and
+    # takes the anchors from tables), so that fraction can exceed 1 and does not
+    # bound the kernel.
     roof = {"bound": "hbm", "achieved": bytes_per_launch / avg_launch_s / 1e9, "peak": hbm_gbs,
             "unit": "GB/s", "peak_source": f"{hbm_src} copy bandwidth (MEASURED_PEAKS.json hbm_gbs)"}
     roof["frac"] = roof["achieved"] / roof["peak"]
@@ -475,9 +475,9 @@ def run_ours(args):
                 "roofline": {"bound": "fp64", "algorithmic_flops_per_pair": pfl,
                              "region_fractions_ABC": [round(f, 4) for f in pfr], "achieved": ptf,
                              "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s", "frac": ptf / FP64_PEAK_TFLOPS,
-                             "note": "the paper's FP64 work per pair against the nominal FP64 peak; above 1 "
-                                     "because region-C pairs take a closed form and most of the rest runs on "
-                                     "the integer pipes (ncu: FP64 pipe 50%, ALU 58% busy)",
+                             "note": "the paper's FP64 work per pair against the nominal FP64 peak; nominal, as the "
+                                     "values are: a pair evaluates an expansion of sum_l c_l F_l that its block "
+                                     "forms, on the integer pipes (ncu: multiply pipe 60% busy), and no F_l",
                              "hbm": "negligible: x, y are re-read from L2/shared memory, 24 B per i"}}
         del xbt, ybt, zbt, cpt
 
@@ -500,7 +500,7 @@ def run_ours(args):
         torch.cuda.synchronize(dev)
         rms = r0.elapsed_time(r1) / args.steps
         # the same batch without a plan: boys_eval_ragged with a grouped-size
-        # workspace (device-built tile table, one launch per kmax)
+        # workspace (device-built tile table, one launch over it)
         wsb = _lib.lib().boys_ragged_workspace_size_grouped(int(km3.size), int(x3.size))
         ws3 = torch.empty(wsb, dtype=torch.uint8, device=dev)
         o3 = torch.empty_like(plan.out)
@@ -522,7 +522,7 @@ def run_ours(args):
                   "fp64_frac": rfl / (rms / 1e3) / 1e12 / FP64_PEAK_TFLOPS, "config": plan.config(),
                   "planless_ms": pl_ms, "planless_vs_plan": pl_ms / rms, "persistent_ms": ps_ms,
                   "launch": "one cudaGraphLaunch: workspace memset + " +
-                            ("one kernel per kmax group (parallel graph branches)" if plan.config()["waves"] == 0
+                            ("one kernel over a table of tiles sorted by kmax" if plan.config()["waves"] == 0
                              else "persistent kernel")}
         plan.close()
         del xt3, ot3, kt3, plan
