@@ -13,7 +13,7 @@
 //
 // What bounds it: the integer multiply pipe, which takes a 32 x 32 -> 64-bit
 // product every clock and SM (and also most moves and adds), at small K; the
-// stores at K = 32 (2^26 arguments of all regions: 2.71 ms, 0.99 of the measured
+// stores at K = 32 (2^26 arguments of all regions: 2.69 ms, 1.00 of the measured
 // copy bandwidth).  All terms of the downward step are positive: it never
 // cancels, one scaling per order serves every lane, and since every lane
 // produces the orders in the same sequence a warp stores whole rows as it goes
@@ -155,7 +155,7 @@ __device__ __forceinline__ double normalise(State& S) {
 // and the same instructions in every region.  Rationals evaluated at x, with their
 // inverse square root, the exponential and region C's inverse square root took
 // about thirty products and the selects of their operands (K = 0, 2^24
-// arguments: 275 us against 105).
+// arguments: 275 us against 84).
 template <int K>
 __device__ __forceinline__ State start(u64 xb, const Local* __restrict__ tab) {
     constexpr int kBitsC = K <= 12 ? 9 : 10;  // index bits of region C: one for the factor of two, log2 of its intervals
