@@ -212,20 +212,29 @@ constexpr int kGroupTile = 128;  // arguments per tile of a table built on the d
 struct GroupHeader {
     Workspace ws;             // error word (the persistent kernel also uses next_tile)
     unsigned count[33];       // tiles per kmax
-    unsigned base[33];        // first tile of each group
-    unsigned cursor[33];      // fill positions
-    unsigned total;           // tiles in all
+    unsigned cursor[33];      // of which are filled
     unsigned overflow;        // 1: the table does not fit, the persistent fallback runs
 };
 constexpr size_t kGroupHeaderBytes = 512;
 static_assert(sizeof(GroupHeader) <= kGroupHeaderBytes, "group header fits its reserved bytes");
 
+// The 33 counts summed up by a warp: lane k gets the first tile of order k + 1.
+__device__ __forceinline__ unsigned group_ends(const GroupHeader* __restrict__ h, unsigned lane) {
+    unsigned run = h->count[lane];
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const unsigned u = __shfl_up_sync(0xffffffffu, run, d);
+        if (lane >= d) run += u;
+    }
+    return run;
+}
+
 __global__ void __launch_bounds__(kMaxBlock, BOYS_RAGGED_MIN_BLOCKS) k_group(
         const double* __restrict__ x, const int64_t* __restrict__ seg_off, double* __restrict__ out,
         const int64_t* __restrict__ out_off, const Tile* __restrict__ tiles, const GroupHeader* __restrict__ h) {
     if (h->overflow) return;
-    const unsigned total = h->total, lane = threadIdx.x & 31;
-    const unsigned base = h->base[lane + 1];  // first tile of kmax lane + 1
+    const unsigned base = group_ends(h, threadIdx.x & 31);  // first tile of kmax lane + 1
+    const unsigned total = __shfl_sync(0xffffffffu, base, 31) + h->count[32];
     for (unsigned i = blockIdx.x; i < total; i += gridDim.x) {
         const unsigned t = total - 1 - i;
         const int k = __popc(__ballot_sync(0xffffffffu, base <= t));
@@ -250,10 +259,10 @@ __global__ void __launch_bounds__(kMaxBlock, BOYS_RAGGED_MIN_BLOCKS) k_group(
 // ------------------------------------ kmax-grouped tiles without a plan
 //
 // With a large enough workspace, boys_eval_ragged builds the table itself, on the
-// device: a count of tiles per kmax, an exclusive scan of the 33 counts (by one warp;
-// one thread after another took 10 us), and a fill in which each segment takes a
+// device: a count of tiles per kmax, and a fill in which each segment takes a
 // contiguous range of its group with one atomic and a warp writes it (the order of
-// tiles inside a group varies, the values do not).  If the table
+// tiles inside a group varies, the values do not).  Every warp sums up the 33 counts
+// for itself.  If the table
 // would exceed the workspace's capacity, the tile kernel returns at once and a
 // persistent launch, gated on that condition, evaluates the batch instead.
 
@@ -273,31 +282,14 @@ __global__ void k_group_count(const int64_t* __restrict__ seg_off, const int32_t
     }
 }
 
-// One warp: lane k takes order k, and all of them order 32.
-__global__ void k_group_scan(GroupHeader* __restrict__ h, unsigned long long capacity) {
-    const unsigned lane = threadIdx.x, mine = h->count[lane];
-    unsigned run = mine;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const unsigned u = __shfl_up_sync(0xffffffffu, run, d);
-        if (lane >= d) run += u;
-    }
-    h->base[lane] = run - mine;
-    h->cursor[lane] = run - mine;
-    if (lane == 31) {
-        const unsigned long long total = (unsigned long long)run + h->count[32];
-        h->base[32] = run;
-        h->cursor[32] = run;
-        h->total = (unsigned)total;
-        h->overflow = total > capacity ? 1u : 0u;
-    }
-}
-
 // A warp per segment: its tiles are written side by side.
 __global__ void k_group_fill(const int64_t* __restrict__ seg_off, const int32_t* __restrict__ seg_kmax, int nseg,
-                             GroupHeader* __restrict__ h, Tile* __restrict__ tiles) {
-    if (h->overflow) return;
-    const unsigned lane = threadIdx.x & 31;
+                             GroupHeader* __restrict__ h, Tile* __restrict__ tiles, unsigned long long capacity) {
+    const unsigned lane = threadIdx.x & 31, ends = group_ends(h, lane);
+    if ((unsigned long long)__shfl_sync(0xffffffffu, ends, 31) + h->count[32] > capacity) {
+        if (blockIdx.x == 0 && threadIdx.x == 0) h->overflow = 1;
+        return;
+    }
     const int64_t warps = (int64_t)gridDim.x * blockDim.x / 32;
     for (int64_t s = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / 32; s < nseg; s += warps) {
         const int64_t len = __ldg(seg_off + s + 1) - __ldg(seg_off + s);
@@ -307,6 +299,7 @@ __global__ void k_group_fill(const int64_t* __restrict__ seg_off, const int32_t*
         unsigned p = 0;
         if (lane == 0) p = atomicAdd(&h->cursor[k], n);
         p = __shfl_sync(0xffffffffu, p, 0);
+        if (k > 0) p += __shfl_sync(0xffffffffu, ends, k - 1);
         for (unsigned t = lane; t < n; t += 32) {
             const int64_t a = (int64_t)t * kGroupTile;
             tiles[p + t] = Tile{(int32_t)s, (int32_t)min((int64_t)kGroupTile, len - a), a};
@@ -370,9 +363,8 @@ boys_status launch_grouped(const double* x, const int64_t* seg_off, const int32_
     if (st != BOYS_OK) return st;
     const int sgrid = (int)std::min<int64_t>((nseg + 255) / 256, (int64_t)sm_count() * 4);
     k_group_count<<<sgrid, 256, 0, stream>>>(seg_off, seg_kmax, nseg, h);
-    k_group_scan<<<1, 32, 0, stream>>>(h, capacity);
     const int fgrid = (int)std::min<int64_t>(((int64_t)nseg * 32 + 255) / 256, (int64_t)sm_count() * 8);
-    k_group_fill<<<fgrid, 256, 0, stream>>>(seg_off, seg_kmax, nseg, h, tiles);
+    k_group_fill<<<fgrid, 256, 0, stream>>>(seg_off, seg_kmax, nseg, h, tiles, capacity);
     st = check_cuda(cudaGetLastError(), "ragged group table");
     k_group<<<group_grid((int64_t)capacity, kGroupTile), kGroupTile, 0, stream>>>(x, seg_off, out, out_off, tiles, h);
     const Config c;
@@ -527,17 +519,16 @@ static boys_status build_tiles(boys_ragged_plan* p, int block) {
     std::vector<ragged::Tile> tab;
     ragged::GroupHeader h = {};
     for (int k = 0; k <= 32; ++k) {
-        h.base[k] = (unsigned)tab.size();
+        const size_t first = tab.size();
         for (int32_t sg = 0; sg < p->nseg; ++sg) {
             if (p->km_host[sg] != k) continue;
             const int64_t len = p->off_host[sg + 1] - p->off_host[sg];
             for (int64_t a = 0; a < len; a += block)
                 tab.push_back(ragged::Tile{sg, (int32_t)std::min<int64_t>(block, len - a), a});
         }
-        h.count[k] = (unsigned)tab.size() - h.base[k];
+        h.count[k] = (unsigned)(tab.size() - first);
     }
     if (tab.size() > 0xFFFFFFFFull) return fail(BOYS_ERR_INVALID_ARG, "boys_ragged_plan_create: too many tiles");
-    h.total = (unsigned)tab.size();
     if (p->header) cudaFree(p->header);
     p->header = nullptr;
     p->tiles = nullptr;
@@ -555,13 +546,12 @@ static boys_status build_tiles(boys_ragged_plan* p, int block) {
     return st;
 }
 
-// Records the batch for configuration c on the capturing stream s: the
-// workspace reset, then the persistent kernel or, for waves == 0, the tile kernel.
+// Records the batch for configuration c on the capturing stream s: the workspace
+// reset and the persistent kernel, or, for waves == 0, the tile kernel alone (the
+// plan's kmax were checked when it was made).
 static boys_status record_launch(boys_ragged_plan* p, const ragged::Config& c, cudaStream_t s) {
     if (c.waves != 0)
         return ragged::launch(c, p->x, p->seg_off, p->seg_kmax, p->nseg, p->out, p->out_off, p->ws, s);
-    boys_status st = check_cuda(cudaMemsetAsync(p->ws, 0, sizeof(ragged::Workspace), s), "ragged workspace reset");
-    if (st != BOYS_OK) return st;
     ragged::k_group<<<ragged::group_grid(p->ntiles, c.block), c.block, 0, s>>>(p->x, p->seg_off, p->out, p->out_off,
                                                                               p->tiles, p->header);
     return check_cuda(cudaGetLastError(), "ragged group launch");
