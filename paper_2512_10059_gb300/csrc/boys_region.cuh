@@ -87,15 +87,15 @@ static __constant__ u64 c_exp[5] = {BOYS_LOCAL_EXP_C0, BOYS_LOCAL_EXP_C1, BOYS_L
                                     BOYS_LOCAL_EXP_C4};
 
 // add + the high half of a b from three partial products, as xf::mulhi3 (at most
-// 2 below the exact high half).  The 32-bit halves are added first, with the carry
-// flag: plain 64-bit adds go to the multiply pipe, at the price of a product each
-// (K = 4: 7% slower).
+// 2 below the exact high half).  The 32-bit halves are added with the carry flag: plain
+// 64-bit adds go to the multiply pipe, at the price of a product each (K = 4, 2^25
+// arguments: 351 us; halves first 356; as 64-bit adds K = 8 3% slower).
 __device__ __forceinline__ u64 mulhi(u64 a, u64 b, u64 add = 0) {
     const unsigned a0 = (unsigned)a, a1 = (unsigned)(a >> 32), b0 = (unsigned)b, b1 = (unsigned)(b >> 32);
     const u64 p = (u64)a1 * b1 + add;
-    unsigned lo = (unsigned)p, hi = (unsigned)(p >> 32), s, c;
-    asm("add.cc.u32 %0, %4, %5;\n\taddc.u32 %1, 0, 0;\n\tadd.cc.u32 %2, %2, %0;\n\taddc.u32 %3, %3, %1;"
-        : "=&r"(s), "=&r"(c), "+r"(lo), "+r"(hi)
+    unsigned lo = (unsigned)p, hi = (unsigned)(p >> 32);
+    asm("add.cc.u32 %0, %0, %2;\n\taddc.u32 %1, %1, 0;\n\tadd.cc.u32 %0, %0, %3;\n\taddc.u32 %1, %1, 0;"
+        : "+r"(lo), "+r"(hi)
         : "r"(__umulhi(a1, b0)), "r"(__umulhi(a0, b1)));
     return (u64)hi << 32 | lo;
 }
