@@ -257,12 +257,14 @@ struct Column {
 };
 
 // Recurrence steps in FP64, the first ones: two instructions and a ready value
-// for 26 on the integer pipes, but at 2 a clock and SM.  Swept on GB300 for every
-// even K with 0 to 12 steps (2^25 arguments): a quarter of the orders is best
-// throughout (K = 32: 3.10 ms with none, 2.95 with 4, 2.77 with 8, 2.88 with 10;
-// K = 16: 886 us with none, 818 with 4, 914 with 6); below K = 6 the conversions
-// cost what the steps save.
-constexpr int fp64_steps(int K) { return K < 6 ? 0 : K / 4; }
+// for 26 on the integer pipes, but at 2 a clock and SM.  Swept on GB300 (2^25
+// arguments, us): about a quarter of the orders, rounded up, to K = 16 (K = 7: 430
+// with 2, 455 with 1; K = 10: 518 with 3, 541 with 2; K = 13: 619 with 4, 627 with 3;
+// K = 16: 731 with 4, 738 with 3, 734 with 5), a fifth above, where the stores take
+// over (K = 24: 1038 with 4, 1044 with 6; K = 32, 2^26: 2692 with 6, 2698 with 8).
+// None below K = 6: one would give 1 % at K = 4 (347 for 352), and the results there
+// are those of the exact integer arithmetic to the last bit.
+constexpr int fp64_steps(int K) { return K < 6 ? 0 : K <= 16 ? (K + 3) / 4 : K < 20 ? 4 : K / 5; }
 
 // F_K, F_{K-1}, ..., F_LAST at a regular x, to out(integral_constant k, value);
 // `tab` is the order's table.
