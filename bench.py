@@ -521,9 +521,9 @@ def run_ours(args):
                   "hbm_gbs": rbytes / (rms / 1e3) / 1e9,
                   "fp64_frac": rfl / (rms / 1e3) / 1e12 / FP64_PEAK_TFLOPS, "config": plan.config(),
                   "planless_ms": pl_ms, "planless_vs_plan": pl_ms / rms, "persistent_ms": ps_ms,
-                  "launch": "one cudaGraphLaunch: workspace memset + " +
+                  "launch": "one cudaGraphLaunch: " +
                             ("one kernel over a table of tiles sorted by kmax" if plan.config()["waves"] == 0
-                             else "persistent kernel")}
+                             else "workspace memset + persistent kernel")}
         plan.close()
         del xt3, ot3, kt3, plan
 
