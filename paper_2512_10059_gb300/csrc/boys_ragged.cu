@@ -542,6 +542,9 @@ static boys_status build_tiles(boys_ragged_plan* p, int block) {
     if (st == BOYS_OK && !tab.empty())
         st = check_cuda(cudaMemcpy(p->tiles, tab.data(), tab.size() * sizeof(ragged::Tile), cudaMemcpyHostToDevice),
                         "plan tile table upload");
+    // A copy from pageable memory may return before its DMA has ended, and the plan's
+    // graph is replayed on streams that do not wait for the default one.
+    if (st == BOYS_OK) st = check_cuda(cudaStreamSynchronize(nullptr), "plan tile table upload");
     if (st == BOYS_OK) p->tiles_block = block;
     return st;
 }
