@@ -48,7 +48,9 @@ constexpr int kNotFinite = -100000;
 // Expansion of w about the right edge in t = 4 (edge - X), t in [0, 1/4]: signed
 // integers, a0..a4 in units of 2^(ex - 62), a5..a8 in 2^14 of those.  The unit follows
 // the interval's own sum |c_l| F_l, so that w keeps its relative accuracy where it is
-// small.
+// small; it holds the weights' scale too, so that y_j meets w itself (a sum of y_j w
+// over the scale overflowed, or ran out of bits, where y and the weights offset each
+// other).
 struct __align__(16) Entry {
     long long a0, a1, a2, a3, a4;
     int a5, a6, a7, a8;
@@ -80,7 +82,11 @@ __device__ __forceinline__ long long level(int t1, int t0, long long u, long lon
     return (long long)((u64)hi << 32 | lo);
 }
 
-// v 2^(ex - 62) as a double (truncated); |ex| < 900.
+// Weights below this are taken up to it in the table and back in the sum: the unit's
+// exponent stays above it less 84 (F_32 at X = 64) and a double's exponent has room.
+constexpr int kMinScale = -900;
+
+// v 2^(ex - 62) as a double (truncated); ex >= kMinScale - 84, the value below 2^1021.
 __device__ __forceinline__ double unit_double(long long v, int ex) {
     const long long sign = v >> 63;
     const u64 a = (u64)(v ^ sign);
@@ -96,7 +102,7 @@ __device__ __forceinline__ double unit_double(long long v, int ex) {
 
 constexpr u64 kOutside = 1ULL << 62;  // 64 in units of 2^-56
 
-// w at X = U 2^-56 < 64 from its interval's expansion, over 2^scale.
+// w at X = U 2^-56 < 64 from its interval's expansion.
 __device__ __forceinline__ double w_table(const Entry* __restrict__ tab, u64 U) {
     const Entry* const e = tab + (int)(U >> 52);
     // edge - X = (2^52 - d) 2^-56 with d = U mod 2^52, and t is four of it
@@ -126,7 +132,7 @@ struct Weighted {
     __device__ __forceinline__ void operator()(std::integral_constant<int, L>, double v) { s = fma(c[L], v, s); }
 };
 
-// w(X) order by order.
+// w(X) order by order.  efx holds the region-C sum's coefficients in units of 2^-fe.
 template <int K>
 __device__ __noinline__ double w_direct(double X, const double* c, const long long* efx, int fe) {
     const u64 xb = region::bits_of(X);
@@ -149,11 +155,11 @@ __device__ __noinline__ double w_direct(double X, const double* c, const long lo
     return xf::to_double(xf::mul(xf::sqrt_pi_over_2(), r)) * fixed_to_double(h, fe);
 }
 
-// The entry of the interval that ends at x = (e + 1) / 16, for weights c scaled to
-// sum |c_l| in [1/2, 1] (or all zero), from S_i = sum_l c_l F_{l+i}(x), i = 0..8.  The
+// The entry of the interval that ends at x = (e + 1) / 16, for weights c 2^scale, c
+// with sum |c_l| in [1/2, 1] (or all zero), from S_i = sum_l c_l F_{l+i}(x), i = 0..8.  The
 // terms from i = 5 on weigh below 2^-26, so single precision serves them.
 template <int K>
-__device__ __noinline__ void expand(int e, const double* c, Entry& E) {
+__device__ __noinline__ void expand(int e, const double* c, int scale, Entry& E) {
     double S[5] = {0, 0, 0, 0, 0}, bound = 0.0;
     float s4[4] = {0, 0, 0, 0};
 #pragma unroll 1
@@ -178,7 +184,7 @@ __device__ __noinline__ void expand(int e, const double* c, Entry& E) {
     E.a6 = (int)__double2ll_rn(ldexp((double)s4[1] * (1.0 / 720), s - 12 - 14));
     E.a7 = (int)__double2ll_rn(ldexp((double)s4[2] * (1.0 / 5040), s - 14 - 14));
     E.a8 = (int)__double2ll_rn(ldexp((double)s4[3] * (1.0 / 40320), s - 16 - 14));
-    E.ex = 62 - s;
+    E.ex = 62 - s + scale;
 }
 
 constexpr int kTileJ = kBlock;
@@ -198,35 +204,35 @@ __global__ void __launch_bounds__(kBlock, 3) k_pairwise(const double* __restrict
     if (t <= K) s_c[t] = __ldg(c + t);
     __syncthreads();
     if (t == 0) {
-        // The binary point of the region-C sum over e_l = c_l (2l-1)!! / 32^l, and the
-        // exponent of sum |c_l|, by which the table's weights are scaled
+        // The exponent of sum |c_l|, by which the weights are scaled, and the binary
+        // point of the region-C sum over e_l = c_l (2l-1)!! / 32^l of the scaled ones
         double se = 0.0, sc = 0.0, f = 1.0;
+        for (int l = 0; l <= K; ++l) sc += fabs(s_c[l]);
+        const bool finite = sc < 0x1p1020;
+        const int scale = finite ? (sc > 0.0 ? ilogb(sc) + 1 : 0) : kNotFinite;
         for (int l = 0; l <= K; ++l) {
-            se += fabs(ldexp(s_c[l] * f, -5 * l));
-            sc += fabs(s_c[l]);
+            s_cn[l] = finite ? ldexp(s_c[l], -scale) : 0.0;
+            se += fabs(ldexp(s_cn[l] * f, -5 * l));
             f *= (double)(2 * l + 1);
         }
-        const bool finite = se < INFINITY && sc < INFINITY;
-        const int fe = finite ? fixed_point_for(se) : kNotFinite;
-        const int scale = finite ? (sc > 0.0 ? ilogb(sc) + 1 : 0) : kNotFinite;
+        const int fe = fixed_point_for(se);
         f = 1.0;
         for (int l = 0; l <= K; ++l) {
-            s_efx[l] = finite ? __double2ll_rn(ldexp(ldexp(s_c[l] * f, -5 * l), fe)) : 0;
-            s_cn[l] = finite ? ldexp(s_c[l], -scale) : 0.0;
+            s_efx[l] = __double2ll_rn(ldexp(ldexp(s_cn[l] * f, -5 * l), fe));
             f *= (double)(2 * l + 1);
         }
-        s_fe = fe;
+        s_fe = finite ? fe - scale : kNotFinite;
         s_scale = scale;
     }
     __syncthreads();
-    const int scale = s_scale;
+    const int scale = s_scale, held = max(scale, kMinScale);
     const bool table = scale != kNotFinite;
     if (table)
-        for (int e = t; e < kEntries; e += kBlock) expand<K>(e, s_cn, s_tab[e]);
+        for (int e = t; e < kEntries; e += kBlock) expand<K>(e, s_cn, held, s_tab[e]);
     const int64_t i = (int64_t)(blockIdx.x / parts) * kBlock + t;
     const double xi = i < n ? __ldg(x + i) : 0.0;
     const u64 ui = table ? to_units(xi) : 0x7FFFFFFFFFFFFFFFULL;
-    double zt = 0.0, zd = 0.0;  // the table's pairs, in units of 2^scale, and the others
+    double zt = 0.0, zd = 0.0;  // the table's pairs, in units of 2^(scale - held), and the others
     const int64_t tiles = (n + kTileJ - 1) / kTileJ;
     const int64_t first = tiles * part / parts, last = tiles * (part + 1) / parts;
     for (int64_t tile = first; tile < last; ++tile) {
@@ -271,7 +277,7 @@ __global__ void __launch_bounds__(kBlock, 3) k_pairwise(const double* __restrict
             else zd = fma(s_y[jj], w_direct<K>(xi + s_x[jj], s_c, s_efx, s_fe), zd);
         }
     }
-    const double zi = table ? ldexp(zt, scale) + zd : zd;
+    const double zi = scale < held && table ? ldexp(zt, scale - held) + zd : zt + zd;
     if (parts == 1) {
         if (i < n) z[i] = zi;
         return;
