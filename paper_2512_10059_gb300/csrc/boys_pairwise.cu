@@ -157,33 +157,35 @@ __device__ __noinline__ double w_direct(double X, const double* c, const long lo
 
 // The entry of the interval that ends at x = (e + 1) / 16, for weights c 2^scale, c
 // with sum |c_l| in [1/2, 1] (or all zero), from S_i = sum_l c_l F_{l+i}(x), i = 0..8.  The
-// terms from i = 5 on weigh below 2^-26, so single precision serves them.
+// sums run from the highest order down, the smallest values first: from 0 up, the sums'
+// rounding reached 10 units of 2^-53 sum |c_l| F_l (K = 32, X > 36).
 template <int K>
 __device__ __noinline__ void expand(int e, const double* c, int scale, Entry& E) {
-    double S[5] = {0, 0, 0, 0, 0}, bound = 0.0;
-    float s4[4] = {0, 0, 0, 0};
+    double S[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, bound = 0.0;
 #pragma unroll 1
-    for (int l = 0; l <= K; ++l) {
+    for (int l = K; l >= 0; --l) {
         const double cl = c[l];
-        const float cf = (float)cl;
         const double* f = &g_grid_f[l][e];
         bound = fma(fabs(cl), __ldg(f), bound);
 #pragma unroll
-        for (int i = 0; i <= 4; ++i) S[i] = fma(cl, __ldg(f + i * kEntries), S[i]);
-#pragma unroll
-        for (int i = 5; i <= 8; ++i) s4[i - 5] = fmaf(cf, (float)__ldg(f + i * kEntries), s4[i - 5]);
+        for (int i = 0; i <= 8; ++i) S[i] = fma(cl, __ldg(f + i * kEntries), S[i]);
     }
     // on the whole interval sum |c_l| F_l <= e^{1/16} bound; its unit keeps |w| below 2^61
     const int s = bound > 0.0 ? 59 - ilogb(bound) : 62;
-    E.a0 = __double2ll_rn(ldexp(S[0], s));
+    // Half of what the cut to a double drops at this size goes in, so that w is
+    // rounded to nearest instead (where the interval stays within a factor of two).
+    const long long a0 = __double2ll_rn(ldexp(S[0], s));
+    const int lead = 63 - __clzll(llabs(a0) | 1);
+    const long long half = lead < 53 ? 0 : 1LL << (lead - 53);
+    E.a0 = a0 < 0 ? a0 - half : a0 + half;
     E.a1 = __double2ll_rn(ldexp(S[1], s - 2));
     E.a2 = __double2ll_rn(ldexp(S[2] * (1.0 / 2), s - 4));
     E.a3 = __double2ll_rn(ldexp(S[3] * (1.0 / 6), s - 6));
     E.a4 = __double2ll_rn(ldexp(S[4] * (1.0 / 24), s - 8));
-    E.a5 = (int)__double2ll_rn(ldexp((double)s4[0] * (1.0 / 120), s - 10 - 14));
-    E.a6 = (int)__double2ll_rn(ldexp((double)s4[1] * (1.0 / 720), s - 12 - 14));
-    E.a7 = (int)__double2ll_rn(ldexp((double)s4[2] * (1.0 / 5040), s - 14 - 14));
-    E.a8 = (int)__double2ll_rn(ldexp((double)s4[3] * (1.0 / 40320), s - 16 - 14));
+    E.a5 = (int)__double2ll_rn(ldexp(S[5] * (1.0 / 120), s - 10 - 14));
+    E.a6 = (int)__double2ll_rn(ldexp(S[6] * (1.0 / 720), s - 12 - 14));
+    E.a7 = (int)__double2ll_rn(ldexp(S[7] * (1.0 / 5040), s - 14 - 14));
+    E.a8 = (int)__double2ll_rn(ldexp(S[8] * (1.0 / 40320), s - 16 - 14));
     E.ex = 62 - s + scale;
 }
 
