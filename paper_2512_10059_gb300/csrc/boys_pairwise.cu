@@ -10,7 +10,8 @@
 // to the last bit of a double), forms the expansions of w to degree 8 about them in
 // shared memory (64 KB, in integers), and a pair is then an index, eight products
 // of a Horner sum and one FMA.  The truncation is below 2^-54 sum |c_l| F_l; the
-// coefficients carry the FP64 rounding that the sum over l had pair by pair.  Bound by
+// coefficients carry the FP64 rounding that the sum over l had pair by pair.  A block
+// whose j have few pairs there expands w at those alone.  Bound by
 // the multiply pipe (17 products and as many other instructions that run there, 31
 // of 48 SM cycles for the 32 pairs of a warp); evaluating the orders for each pair took
 // 255 cycles where x is sorted and the chip full (k = 12: n = 65536 155 to 21 ms,
@@ -100,11 +101,23 @@ __device__ __forceinline__ double unit_double(long long v, int ex) {
     return __hiloint2double((int)(top | ((unsigned)(sign >> 32) & 0x80000000u)), (int)region::shift_right(l, h, 10));
 }
 
+// (2l-1)!! / 32^l
+struct Closed {
+    double v[33];
+    constexpr Closed() : v{} {
+        double f = 1.0, p = 1.0;
+        for (int l = 0; l <= 32; ++l, p /= 32.0) {
+            v[l] = f * p;
+            f *= (double)(2 * l + 1);
+        }
+    }
+};
+static __constant__ Closed c_closed;
+
 constexpr u64 kOutside = 1ULL << 62;  // 64 in units of 2^-56
 
 // w at X = U 2^-56 < 64 from its interval's expansion.
-__device__ __forceinline__ double w_table(const Entry* __restrict__ tab, u64 U) {
-    const Entry* const e = tab + (int)(U >> 52);
+__device__ __forceinline__ double w_entry(const Entry* __restrict__ e, u64 U) {
     // edge - X = (2^52 - d) 2^-56 with d = U mod 2^52, and t is four of it
     const u64 tq = ~(U << 12) >> 2;  // t in Q64
     const int t0 = (int)(unsigned)tq, t1 = (int)((unsigned)(tq >> 32) + ((unsigned)tq >> 31));
@@ -159,16 +172,24 @@ __device__ __noinline__ double w_direct(double X, const double* c, const long lo
 // with sum |c_l| in [1/2, 1] (or all zero), from S_i = sum_l c_l F_{l+i}(x), i = 0..8.  The
 // sums run from the highest order down, the smallest values first: from 0 up, the sums'
 // rounding reached 10 units of 2^-53 sum |c_l| F_l (K = 32, X > 36).
-template <int K>
+// kLanes > 1: that many neighbouring lanes share an entry, every kLanes-th order each.
+template <int K, int kLanes>
 __device__ __noinline__ void expand(int e, const double* c, int scale, Entry& E) {
     double S[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, bound = 0.0;
 #pragma unroll 1
-    for (int l = K; l >= 0; --l) {
+    for (int l = K - (int)(threadIdx.x & (kLanes - 1)); l >= 0; l -= kLanes) {
         const double cl = c[l];
         const double* f = &g_grid_f[l][e];
         bound = fma(fabs(cl), __ldg(f), bound);
 #pragma unroll
         for (int i = 0; i <= 8; ++i) S[i] = fma(cl, __ldg(f + i * kEntries), S[i]);
+    }
+#pragma unroll
+    for (int d = 1; d < kLanes; d <<= 1) {
+        const unsigned group = ((1u << kLanes) - 1) << (threadIdx.x & 31 & ~(kLanes - 1));
+        bound += __shfl_xor_sync(group, bound, d);
+#pragma unroll
+        for (int i = 0; i <= 8; ++i) S[i] += __shfl_xor_sync(group, S[i], d);
     }
     // on the whole interval sum |c_l| F_l <= e^{1/16} bound; its unit keeps |w| below 2^61
     const int s = bound > 0.0 ? 59 - ilogb(bound) : 62;
@@ -189,7 +210,36 @@ __device__ __noinline__ void expand(int e, const double* c, int scale, Entry& E)
     E.ex = 62 - s + scale;
 }
 
+// w at X = U 2^-56 < 64 without the table: the interval's entry for this pair alone.
+template <int K, int kLanes>
+__device__ __noinline__ double w_alone(u64 U, const double* c, int scale) {
+    Entry E;
+    expand<K, kLanes>((int)(U >> 52), c, scale, E);
+    return w_entry(&E, U);
+}
+
 constexpr int kTileJ = kBlock;
+// A block forms the table if more than this many of its j have pairs in it; the pairs
+// of fewer j are expanded one by one.  Every block used to form it: a call of one pair
+// took 55 us at k = 12 and 110 at k = 32 (10 and 14 now), and one whose pairs all
+// lie beyond it, n = 256 with x on [32, 300], 275 at k = 12 (35 now).  n = 32, 48, 64
+// (4, 6, 8 j a block) by the table and by pairs, us: k = 0 27, 28, 29 and 19, 25, 29;
+// k = 12 57, 59, 59 and 43, 62, 80; k = 32 112, 113, 113 and 88, 127, 165.
+#ifndef BOYS_PAIRWISE_TABLE_J
+#define BOYS_PAIRWISE_TABLE_J 5
+#endif
+// Up to kFewRows rows, kFewLanes threads serve one row (an FP64 instruction of a warp
+// costs 64 clocks of its quarter of the SM however few of its lanes are in use: n = 8, k
+// = 32: 47 us with one, 16 with four), and the table is never formed.
+constexpr int kFewRows = 8, kFewLanes = 4;
+static_assert(kFewRows * kFewLanes <= 32 && BOYS_PAIRWISE_TABLE_J >= 2, "few rows share a warp, at most two j a block");
+
+// The sum of a warp's values, in every lane.
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
+    return v;
+}
 
 template <int K>
 __global__ void __launch_bounds__(kBlock, 3) k_pairwise(const double* __restrict__ x, const double* __restrict__ y,
@@ -200,58 +250,76 @@ __global__ void __launch_bounds__(kBlock, 3) k_pairwise(const double* __restrict
     __shared__ u64 s_u[kTileJ];
     __shared__ long long s_efx[K + 1];
     __shared__ int s_fe, s_scale;
+    __shared__ unsigned s_low[kBlock / 32];
     const cg::cluster_group cluster = cg::this_cluster();
     const int parts = (int)cluster.num_blocks(), part = (int)cluster.block_rank();
     const int t = threadIdx.x;
     if (t <= K) s_c[t] = __ldg(c + t);
     __syncthreads();
-    if (t == 0) {
+    if (t < 32) {
         // The exponent of sum |c_l|, by which the weights are scaled, and the binary
-        // point of the region-C sum over e_l = c_l (2l-1)!! / 32^l of the scaled ones
-        double se = 0.0, sc = 0.0, f = 1.0;
-        for (int l = 0; l <= K; ++l) sc += fabs(s_c[l]);
+        // point of the region-C sum over e_l = c_l (2l-1)!! / 32^l of the scaled ones;
+        // lane t has the orders t and t + 32
+        double sc = 0.0, se = 0.0, e[2] = {0.0, 0.0};
+        for (int l = t; l <= K; l += 32) sc += fabs(s_c[l]);
+        sc = warp_sum(sc);
         const bool finite = sc < 0x1p1020;
         const int scale = finite ? (sc > 0.0 ? ilogb(sc) + 1 : 0) : kNotFinite;
-        for (int l = 0; l <= K; ++l) {
-            s_cn[l] = finite ? ldexp(s_c[l], -scale) : 0.0;
-            se += fabs(ldexp(s_cn[l] * f, -5 * l));
-            f *= (double)(2 * l + 1);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int l = t + 32 * q;
+            if (l > K) break;
+            const double cn = finite ? ldexp(s_c[l], -scale) : 0.0;
+            s_cn[l] = cn;
+            e[q] = cn * c_closed.v[l];
+            se += fabs(e[q]);
         }
+        se = warp_sum(se);
         const int fe = fixed_point_for(se);
-        f = 1.0;
-        for (int l = 0; l <= K; ++l) {
-            s_efx[l] = __double2ll_rn(ldexp(ldexp(s_cn[l] * f, -5 * l), fe));
-            f *= (double)(2 * l + 1);
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+            if (t + 32 * q <= K) s_efx[t + 32 * q] = __double2ll_rn(ldexp(e[q], fe));
+        if (t == 0) {
+            s_fe = finite ? fe - scale : kNotFinite;
+            s_scale = scale;
         }
-        s_fe = finite ? fe - scale : kNotFinite;
-        s_scale = scale;
     }
+    const bool few = n <= kFewRows;
+    const int64_t i = few ? t / kFewLanes : (int64_t)(blockIdx.x / parts) * kBlock + t;
+    const bool row = i < n, writes = row && !(few && t % kFewLanes);
+    const double xi = row ? __ldg(x + i) : INFINITY;
+    const int64_t first = n * part / parts, last = n * (part + 1) / parts;
+    // Whether to form the table: j that have a pair in it are those with x_j below 64
+    // less the smallest x_i (by the high words of both, so some just above count too).
+    const unsigned low = __reduce_min_sync(0xffffffffu, (unsigned)(to_units(xi) >> 32));
+    if ((t & 31) == 0) s_low[t / 32] = low;
     __syncthreads();
     const int scale = s_scale, held = max(scale, kMinScale);
-    const bool table = scale != kNotFinite;
+    unsigned lowest = s_low[0];
+#pragma unroll
+    for (int w = 1; w < kBlock / 32; ++w) lowest = min(lowest, s_low[w]);
+    int inside = 0;
+    for (int64_t j0 = first; j0 < last && inside <= BOYS_PAIRWISE_TABLE_J && scale != kNotFinite; j0 += kBlock)
+        inside += __syncthreads_count(j0 + t < last && lowest + (unsigned)(to_units(__ldg(x + j0 + t)) >> 32) < (unsigned)(kOutside >> 32));
+    const bool table = inside > BOYS_PAIRWISE_TABLE_J;
     if (table)
-        for (int e = t; e < kEntries; e += kBlock) expand<K>(e, s_cn, held, s_tab[e]);
-    const int64_t i = (int64_t)(blockIdx.x / parts) * kBlock + t;
-    const double xi = i < n ? __ldg(x + i) : 0.0;
-    const u64 ui = table ? to_units(xi) : 0x7FFFFFFFFFFFFFFFULL;
+        for (int e = t; e < kEntries; e += kBlock) expand<K, 1>(e, s_cn, held, s_tab[e]);
+    const u64 ui = scale != kNotFinite ? to_units(xi) : 0x7FFFFFFFFFFFFFFFULL;
     double zt = 0.0, zd = 0.0;  // the table's pairs, in units of 2^(scale - held), and the others
-    const int64_t tiles = (n + kTileJ - 1) / kTileJ;
-    const int64_t first = tiles * part / parts, last = tiles * (part + 1) / parts;
-    for (int64_t tile = first; tile < last; ++tile) {
-        const int64_t j0 = tile * kTileJ;
+    for (int64_t j0 = first; j0 < last; j0 += kTileJ) {
         __syncthreads();
-        if (j0 + t < n) {
+        if (j0 + t < last) {
             const double xj = __ldg(x + j0 + t);
             s_x[t] = xj;
             s_u[t] = to_units(xj);
             s_y[t] = __ldg(y + j0 + t);
         }
         __syncthreads();
-        const int jn = (int)min((int64_t)kTileJ, n - j0);
+        const int jn = row ? (int)min((int64_t)kTileJ, last - j0) : 0;
         // Two pairs at a time, the products of one filling the waits of the other (n =
         // 65536, k = 12: 22.4 ms with one, 21.1 with two, 20.9 with four).
         int jj = 0;
-        for (; jj + 2 <= jn; jj += 2) {
+        for (; table && jj + 2 <= jn; jj += 2) {
             u64 U[2], all = 0;
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
@@ -261,32 +329,34 @@ __global__ void __launch_bounds__(kBlock, 3) k_pairwise(const double* __restrict
             if (all < kOutside) {
                 double w[2];
 #pragma unroll
-                for (int q = 0; q < 2; ++q) w[q] = w_table(s_tab, U[q]);
+                for (int q = 0; q < 2; ++q) w[q] = w_entry(s_tab + (int)(U[q] >> 52), U[q]);
 #pragma unroll
                 for (int q = 0; q < 2; ++q) zt = fma(s_y[jj + q], w[q], zt);
             } else {
 #pragma unroll 1
                 for (int q = 0; q < 2; ++q) {
                     const u64 V = ui + s_u[jj + q];
-                    if (V < kOutside) zt = fma(s_y[jj + q], w_table(s_tab, V), zt);
+                    if (V < kOutside) zt = fma(s_y[jj + q], w_entry(s_tab + (int)(V >> 52), V), zt);
                     else zd = fma(s_y[jj + q], w_direct<K>(xi + s_x[jj + q], s_c, s_efx, s_fe), zd);
                 }
             }
         }
         for (; jj < jn; ++jj) {
             const u64 V = ui + s_u[jj];
-            if (V < kOutside) zt = fma(s_y[jj], w_table(s_tab, V), zt);
+            if (V < kOutside)
+                zt = fma(s_y[jj], table ? w_entry(s_tab + (int)(V >> 52), V) : few ? w_alone<K, kFewLanes>(V, s_cn, held)
+                                                                                 : w_alone<K, 1>(V, s_cn, held), zt);
             else zd = fma(s_y[jj], w_direct<K>(xi + s_x[jj], s_c, s_efx, s_fe), zd);
         }
     }
-    const double zi = scale < held && table ? ldexp(zt, scale - held) + zd : zt + zd;
+    const double zi = scale < held ? ldexp(zt, scale - held) + zd : zt + zd;
     if (parts == 1) {
-        if (i < n) z[i] = zi;
+        if (writes) z[i] = zi;
         return;
     }
     s_z[t] = zi;
     cluster.sync();
-    if (part == 0 && i < n) {
+    if (part == 0 && writes) {
         double sum = zi;
         for (int r = 1; r < parts; ++r) sum += cluster.map_shared_rank(s_z, r)[t];
         z[i] = sum;
@@ -316,9 +386,9 @@ BOYS_API boys_status boys_pairwise(const double* x, const double* y, int64_t n, 
     static constexpr auto t = pairwise_table(std::make_integer_sequence<int, 33>{});
     const int64_t rows = (n + kBlock - 1) / kBlock;
     // As many parts (a power of two) as bring the grid to eight blocks per SM, as long
-    // as each keeps a tile.
+    // as each keeps one j.
     int parts = 1;
-    while (parts < kMaxCluster && rows * parts < (int64_t)sm_count() * 8 && 2 * parts <= rows) parts *= 2;
+    while (parts < kMaxCluster && rows * parts < (int64_t)sm_count() * 8 && 2 * parts <= n) parts *= 2;
     if (rows * parts > 0x7fffffff) return fail(BOYS_ERR_INVALID_ARG, "boys_pairwise: grid too large");
     const size_t smem = sizeof(Entry) * kEntries;
     boys_status st = check_cuda(cudaFuncSetAttribute((const void*)t[k], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
