@@ -220,8 +220,9 @@ __device__ __forceinline__ u64 bits_of(double x) {
 __device__ __forceinline__ bool regular(u64 xb) { return xb <= kBitsTwo28; }  // negative numbers and NaN lie above
 
 // Large, infinite and invalid arguments: rare, so a rolled loop, upward: to
-// out(k, value) with a run-time k.  F_k below the normal range flushes to zero, +inf
-// gives 0, an invalid argument NaN.
+// out(k, value) with a run-time k.  F_k below the normal range becomes subnormal (every
+// order alike: the former FP64 steps gave these values, the integer ones 0), +inf gives
+// 0, an invalid argument NaN.
 template <class Out>
 __device__ __forceinline__ void eval_other(int K, double x, Out&& out) {
     const long long xb = __double_as_longlong(x);
@@ -231,7 +232,7 @@ __device__ __forceinline__ void eval_other(int K, double x, Out&& out) {
     const xf::Xf R = xf::mul(xf::Xf{r.m, r.e - 1}, r);
 #pragma unroll 1
     for (int j = 0; j <= K; ++j) {
-        out(j, valid ? xf::to_double(y) : __longlong_as_double(0x7FF8000000000000LL));
+        out(j, valid ? xf::to_double_gradual(y) : __longlong_as_double(0x7FF8000000000000LL));
         y = xf::mul_norm(xf::mul_raw(xf::odd(j), y), R);
     }
 }

@@ -109,6 +109,12 @@ __device__ __forceinline__ unsigned long long shr_u64(unsigned long long a, int 
     asm("shr.b64 %0, %1, %2;" : "=l"(r) : "l"(a), "r"(n));
     return r;
 }
+
+// Xf -> double with gradual underflow (cut to a unit of 2^-1074).
+__device__ __forceinline__ double to_double_gradual(Xf v) {
+    return __longlong_as_double((long long)(v.e < -1022 ? shr_u64(v.m, -1011 - v.e) : double_bits(v)));
+}
+
 // a b for an operand a with at most four leading zeros (a raw product) and a
 // normalised b, renormalised by a 32-bit leading-zero count of the high
 // word (the product's leading bit lies in bits 57..63; zero stays zero).
