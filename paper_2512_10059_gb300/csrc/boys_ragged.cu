@@ -386,6 +386,11 @@ const std::vector<Config>& candidates() {
     return c;
 }
 
+// Part of the cache's keys: raised whenever a shape stands for other kernels than
+// before, so that a stored choice among the former ones is made anew (2: waves = 0 is one
+// launch over a table of tiles, 512 segments 27 to 11 us; it was a launch per kmax).
+constexpr int kShapes = 2;
+
 std::string device_key() {
     int dev = 0, drv = 0;
     cudaGetDevice(&dev);
@@ -393,8 +398,8 @@ std::string device_key() {
     cudaDeviceProp p;
     if (cudaGetDeviceProperties(&p, dev) != cudaSuccess) return "unknown";
     char buf[512];
-    snprintf(buf, sizeof(buf), "%.200s|sm%d%d|%dSM|drv%d|lib%d", p.name, p.major, p.minor, p.multiProcessorCount, drv,
-             boys_version());
+    snprintf(buf, sizeof(buf), "%.200s|sm%d%d|%dSM|drv%d|lib%d|shapes%d", p.name, p.major, p.minor, p.multiProcessorCount, drv,
+             boys_version(), kShapes);
     for (char* q = buf; *q; ++q)
         if (*q == ' ') *q = '_';
     return buf;

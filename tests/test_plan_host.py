@@ -9,6 +9,7 @@ default stream.  Device memory is host memory; kernels do not run.
 """
 import ctypes
 import os
+import shutil
 import subprocess
 
 import numpy as np
@@ -135,3 +136,23 @@ def test_tile_table_is_on_the_device_before_a_replay(host, monkeypatch):
     monkeypatch.setenv("BOYS_FORCE_CONFIG", "128,1,0")
     assert _create(host, 2) == (128, 1, 0)
     assert host.fake_pending() == 0
+
+
+def test_stored_shapes_of_former_kernels_are_not_taken(host, tmp_path, monkeypatch):
+    """A cache file written when the shapes stood for other kernels (its keys name
+    the library's version only) is passed over; one written now is taken."""
+    cache = tmp_path / "tune.txt"
+    cache.write_text("Stand_In|sm103|152SM|drv13000|lib100|n2^10|seg4|w23.41 256 2 2\n")
+    monkeypatch.setenv("BOYS_AUTOTUNE_CACHE", str(cache))
+    best = _create(host, 1)
+    assert best == (64, 1, 1) and host.fake_launches() > 0  # every shape takes 1 ms here, the first one wins
+    lines = cache.read_text().splitlines()
+    assert len(lines) == 2 and lines[1].split()[1:] == ["64", "1", "1"]
+    cache.write_text(lines[1].replace(" 64 1 1", " 128 1 0") + "\n")
+    again = tmp_path / "again.so"
+    shutil.copy(host._name, again)
+    fresh = ctypes.CDLL(str(again))
+    for f in ("boys_ragged_plan_create", "boys_ragged_plan_config", "boys_ragged_plan_destroy"):
+        getattr(fresh, f).restype, getattr(fresh, f).argtypes = _lib.SIGNATURES[f]
+    fresh.fake_launches.restype = ctypes.c_long
+    assert _create(fresh, 1) == (128, 1, 0) and fresh.fake_launches() == 0
