@@ -19,7 +19,12 @@ _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", lambda dev: torch.c
 
 
 def _stream_handle(t: torch.Tensor, stream=None) -> int:
-    return int(stream.cuda_stream) if stream is not None else _raw_stream(t.get_device())
+    if stream is not None:
+        return int(stream.cuda_stream)
+    dev = t.get_device()
+    if dev < 0:  # the raw call would take it for the current device
+        raise ValueError(f"Expected a cuda device, but got: {t.device}")
+    return _raw_stream(dev)
 
 
 def _require(t: torch.Tensor, name: str, dtype=torch.float64):
