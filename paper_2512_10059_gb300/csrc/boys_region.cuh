@@ -271,10 +271,11 @@ constexpr int fp64_steps(int K) { return K < 6 ? 0 : K <= 16 ? (K + 3) / 4 : K <
 // `tab` is the order's table.
 //
 // A step, with u the scale of y: T = X y / 2^64 + (Em >> n) is (2l+1) F_l 2^(u-6), its
-// second term free in the product's accumulator, and y = T kappa_l / 2^64.  T stays
-// below 0.56 2^64 and above 2^56 (checked over A and B for every K by the integer
-// model of the tests; in C T < 2^63), so each value carries at least 53.9 correct bits
-// before it is cut to a double's.
+// second term free in the product's accumulator, and y = T kappa_l / 2^64.  T / 2^64 is
+// below (2x + e^{-x} / F_{l+1}) / 128, at most 0.556 in A and B (l = 31, x -> x_1), and
+// below a half in C; it is above 2^56.  A value of the integer steps is within 2^-53
+// of itself before it is cut to a double (the tests' integer model: 2^-53.6 at most,
+// order 0 of K = 31 just above x = 32); an FP64 step adds two roundings of 2^-53.
 template <int K, int NF = fp64_steps(K), int LAST = 0, class Out>
 __device__ __forceinline__ void eval_regular(u64 xb, const Local* __restrict__ tab, Out&& out) {
     const double x = __longlong_as_double((long long)xb);
