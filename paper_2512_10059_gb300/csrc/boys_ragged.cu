@@ -366,6 +366,7 @@ boys_status launch_grouped(const double* x, const int64_t* seg_off, const int32_
     const int fgrid = (int)std::min<int64_t>(((int64_t)nseg * 32 + 255) / 256, (int64_t)sm_count() * 8);
     k_group_fill<<<fgrid, 256, 0, stream>>>(seg_off, seg_kmax, nseg, h, tiles, capacity);
     st = check_cuda(cudaGetLastError(), "ragged group table");
+    if (st != BOYS_OK) return st;
     k_group<<<group_grid((int64_t)capacity, kGroupTile), kGroupTile, 0, stream>>>(x, seg_off, out, out_off, tiles, h);
     const Config c;
     kernel_for(c.xpt)<<<grid_size(c), c.block, 0, stream>>>(x, seg_off, seg_kmax, nseg, out, out_off, &h->ws, &h->overflow);

@@ -29,8 +29,11 @@ static void land() {
     for (auto& c : pending) memcpy(c.dst, c.bytes.data(), c.bytes.size());
     pending.clear();
 }
+static int fail_in;  // the launch that fails, counted from here on (0: none)
+static cudaError_t last = cudaSuccess;
 #define OK return cudaSuccess
 extern "C" {
+void fake_fail(int launch) { fail_in = launch; }
 long fake_pending() { return (long)pending.size(); }
 long fake_launches() { return launches; }
 long fake_early() { return early; }
@@ -40,7 +43,9 @@ void __cudaUnregisterFatBinary(void**) {}
 void __cudaRegisterFunction(void**, const char*, char*, const char*, int, void*, void*, void*, void*, int*) {}
 void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int) {}
 cudaError_t __cudaGetKernel(void** k, const void* f) { *k = (void*)f; OK; }
-cudaError_t __cudaLaunchKernel(void*, dim3, dim3, void**, size_t, void*) { OK; }
+cudaError_t __cudaLaunchKernel(void*, dim3, dim3, void**, size_t, void*) {
+    return fail_in > 0 && --fail_in == 0 ? last = cudaErrorLaunchOutOfResources : cudaSuccess;
+}
 unsigned __cudaPushCallConfiguration(dim3, dim3, size_t, void*) { return 0; }
 cudaError_t __cudaPopCallConfiguration(dim3* g, dim3* b, size_t* m, void* s) {
     *g = *b = dim3(1); *m = 0; *(void**)s = nullptr; OK;
@@ -61,7 +66,7 @@ cudaError_t cudaMemcpyFromSymbolAsync(void*, const void*, size_t, size_t, cudaMe
 cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t) { memset(p, v, n); OK; }
 cudaError_t cudaGetSymbolAddress(void** p, const void* s) { *p = (void*)s; OK; }
 cudaError_t cudaGetDevice(int* d) { *d = 0; OK; }
-cudaError_t cudaGetLastError() { OK; }
+cudaError_t cudaGetLastError() { cudaError_t e = last; last = cudaSuccess; return e; }
 const char* cudaGetErrorName(cudaError_t) { return "error"; }
 const char* cudaGetErrorString(cudaError_t) { return "error"; }
 cudaError_t cudaDriverGetVersion(int* v) { *v = 13000; OK; }
@@ -156,3 +161,19 @@ def test_stored_shapes_of_former_kernels_are_not_taken(host, tmp_path, monkeypat
         getattr(fresh, f).restype, getattr(fresh, f).argtypes = _lib.SIGNATURES[f]
     fresh.fake_launches.restype = ctypes.c_long
     assert _create(fresh, 1) == (128, 1, 0) and fresh.fake_launches() == 0
+
+
+def test_a_failed_launch_is_reported(host):
+    """boys_eval_ragged on a grouped workspace: two launches for the table, one over it and
+    the gated persistent one; whichever fails, the call says so."""
+    _lib.lib()
+    call = host.boys_eval_ragged
+    call.restype, call.argtypes = _lib.SIGNATURES["boys_eval_ragged"]
+    off, km, oo = np.array([0, 5, 300], np.int64), np.array([2, 7], np.int32), np.zeros(2, np.int64)
+    ws = np.zeros(130, np.complex128)  # 16-byte elements: aligned as a workspace is
+    args = (0x1000, off.ctypes.data, km.ctypes.data, 2, 0x1000, oo.ctypes.data, ws.ctypes.data, ws.nbytes, None)
+    assert ws.ctypes.data % 16 == 0 and call(*args) == 0
+    for launch in (1, 2, 3, 4):
+        host.fake_fail(launch)
+        assert call(*args) == 4, launch
+        assert call(*args) == 0
