@@ -60,7 +60,7 @@ HBM_FALLBACK_GBS = 6800.0
 # (profiles/k_eval_f64_kmax32_eri_mixture.md), scaled to the launch by the
 # arguments it processes.  Valid only for the kernel sources it was taken on:
 # the bench reports traffic null whenever their SHA-256 differs.
-TRAFFIC_CAPTURE = {"bytes_per_x": 257.40, "sources_sha256": "05242cbc4932f8304a4afe60479ec957b87bd0a9bc969db831378edb8c2b2b82"}
+TRAFFIC_CAPTURE = {"bytes_per_x": 257.14, "sources_sha256": "1779eaf727ff8e40a21593be5f53cdd0a051edd8f2cb5f2fbaf0e1d8da99a13d"}
 KERNEL_SOURCES = ("boys_fp64.cu", "boys_region.cuh", "gen_local.py", "gen_coeffs_fixed.py", "boys_coeffs_fp64.h",
                   "boys_xf.cuh", "boys_xf_consts.h", "boys_internal.h", "boys_abi.cu")
 

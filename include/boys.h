@@ -209,11 +209,17 @@ void boys_ragged_plan_destroy(boys_ragged_plan* plan);
 /*
  * The paper's benchmark workload (Section III, Algorithm 2):
  *   z[i] = sum_{l=0}^{k} c[l] * sum_{j=0}^{n-1} F_l(x[i] + x[j]) * y[j]
- * for every i, F_l by the three-region Algorithm 1 in FP64 accuracy.
+ * for every i, in FP64 accuracy.
  *   x, y, z [n]; c [k+1]; 0 <= k <= 32; n <= 2^40.
- * Work is n^2 (k+1) evaluations.  Sorting x ascending (permuting y alongside)
- * keeps each warp's arguments in one region and is several times faster; the
- * result is the same up to summation rounding.
+ * For X = x[i] + x[j] < 64 (x[i], x[j] >= 0) the n^2 pairs take w(X) = sum_l c[l]
+ * F_l(X) from expansions about values of the definition (each pair within 2^-50
+ * sum_l |c[l]| F_l(X)), which a block forms once for all its pairs or, where it has
+ * few, pair by pair; other pairs, and weights that are not finite or whose sum
+ * |c[l]| reaches 2^1020, take F_0..F_k by the three-region Algorithm 1.
+ * Products w y[j] are formed as they are, so that y and c may be of any size as
+ * long as these stay in range.  Sorting x ascending (permuting y alongside) keeps
+ * the pairs of a warp near one interval, without shared-memory bank conflicts
+ * (2.6 times faster at n = 2^17); the result is the same up to summation rounding.
  */
 boys_status boys_pairwise(const double* x, const double* y, int64_t n, const double* c, int k, double* z,
                           void* stream);

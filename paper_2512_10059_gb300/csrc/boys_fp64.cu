@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(kBlock, BOYS_STORED_MIN_BLOCKS) k_eval_f64(con
 }
 
 // The fused consumer is bound by the FP64 pipe: kmax FMAs an argument at 2 a clock
-// and SM (kmax 32, 2^24 arguments: 853 us of the 886), so every step of the recurrence
+// and SM (kmax 32, 2^24 arguments: 853 us of the 880), so every step of the recurrence
 // stays on the integer pipes, and so does everything else (with two more FP64
 // instructions an argument, the factor -2 and a comparison, 964 us).  8 blocks per SM
 // suffice (8, 10, 12, 16 blocks: within 1%).

@@ -17,7 +17,7 @@ namespace {
 constexpr int kBlock = 128;
 
 // The sum is kmax + 1 FMAs an argument on the FP64 pipe, at 2 a clock and SM (kmax
-// 16, 2^24 arguments: 453 us of about 500; 561 with two more FP64 instructions, 958 with
+// 16, 2^24 arguments: 453 us of the 486; 561 with two more FP64 instructions, 958 with
 // the recurrence that served all regions), so every step of the recurrence stays on
 // the integer pipes.  8 to 16 blocks per SM are within 1%.
 #ifndef BOYS_GRAD_MIN_BLOCKS

@@ -1,7 +1,6 @@
 // The paper's benchmark workload (Section III, Algorithm 2):
-//     z_i = sum_{l=0}^{k} c_l sum_{j=0}^{n-1} F_l(x_i + x_j) y_j,
-// with the three-region Algorithm 1 for every F_l (Algorithm 2 as printed has
-// no region C although x_i + x_j reaches 60; the three-region method is used).
+//     z_i = sum_{l=0}^{k} c_l sum_{j=0}^{n-1} F_l(x_i + x_j) y_j.
+// (Algorithm 2 as printed has no region C although x_i + x_j reaches 60.)
 //
 // The weights are the same for all n^2 pairs, so a pair needs one function of one
 // variable, w(X) = sum_l c_l F_l(X).  Since dF_l/dX = -F_{l+1}, its Taylor
@@ -13,12 +12,12 @@
 // coefficients carry the FP64 rounding that the sum over l had pair by pair.  A block
 // whose j have few pairs there expands w at those alone.  Bound by
 // the multiply pipe (17 products and as many other instructions that run there, 31
-// of 48 SM cycles for the 32 pairs of a warp); evaluating the orders for each pair took
-// 255 cycles where x is sorted and the chip full (k = 12: n = 65536 155 to 21 ms,
-// n = 2^17 530 to 75 ms).
+// of 52 SM cycles for the 32 pairs of a warp); evaluating the orders for each pair took
+// 255 cycles where x is sorted and the chip full (k = 12: n = 65536 156 to 21 ms,
+// n = 2^17 530 to 73 ms).
 //
-// Pairs with X >= 64 or invalid or infinite X, and all pairs where the weights are not
-// finite, are evaluated order by order: in region C w = F_0 sum_l e_l t^l, e_l = c_l
+// Pairs with X >= 64, with a negative, invalid or infinite argument, and all pairs where
+// the weights are not finite (or near the largest double), are evaluated order by order: in region C w = F_0 sum_l e_l t^l, e_l = c_l
 // (2l-1)!! / 32^l, t = 16 / X, as a fixed-point Horner sum (its partial sums are bounded
 // by sum|e_l|); elsewhere by the downward recurrence of boys_region.cuh and FP64 FMAs.
 //

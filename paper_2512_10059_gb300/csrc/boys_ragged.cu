@@ -1,7 +1,10 @@
 // Ragged batches: many segments, each with its own kmax (e.g. the shell
-// quartets of an ERI batch, kmax_s = la+lb+lc+ld), in ONE persistent launch.
+// quartets of an ERI batch, kmax_s = la+lb+lc+ld).  Two ways to cut the work: flat
+// tiles that a persistent kernel takes from a counter (a 256-byte workspace, the
+// no-alloc entry point, some plans, and where a tile table does not fit), or a table
+// of one-segment tiles sorted by kmax (larger workspaces, most plans; further below).
 //
-// Work decomposition: the concatenated argument array x[0, total) is cut into
+// Flat tiles: the concatenated argument array x[0, total) is cut into
 // flat tiles of blockDim*XPT arguments; resident CTAs take tiles from a
 // global atomic counter (the only scratch memory) until none are left, which
 // balances the very uneven per-argument cost of different kmax.  A thread
@@ -32,9 +35,11 @@
 namespace boys {
 namespace ragged {
 constexpr int kMaxBlock = 256;
-// Resident blocks of kMaxBlock threads per SM: 8 caps the kernels at 32 registers,
-// which every order's evaluation fits (4096 segments at mean kmax 4.07, 3.5e7
-// arguments: 560 us with 8, 612 with 6, 742 with 4).
+// Resident blocks of kMaxBlock threads per SM: 8 caps the kernels at 32 registers.
+// The tile kernel spills one register there; the persistent one 8 (two arguments a
+// thread: 15), its out-of-line evaluations one or two from order 6 on, and it is
+// the fastest all the same (4096 segments at mean kmax 4.07, 3.5e7 arguments:
+// 560 us with 8, 612 with 6, 742 with 4).
 #ifndef BOYS_RAGGED_MIN_BLOCKS
 #define BOYS_RAGGED_MIN_BLOCKS 8
 #endif
@@ -179,7 +184,7 @@ __global__ void __launch_bounds__(kMaxBlock, BOYS_RAGGED_MIN_BLOCKS) k_ragged(co
 // launch walks the table, largest kmax first.  A tile's kmax is the same for the
 // whole block, so the block takes one order's evaluation -- the stored mode's, same
 // bits -- with no segment search and no loop over the kmax of a warp.  All orders
-// fit in 32 registers, so one kernel holds them all at full occupancy.  One kernel
+// fit in 32 registers but for one spill, so one kernel holds them all at full occupancy.  One kernel
 // per kmax, as parallel graph branches of a plan or a chain of programmatic
 // dependents without one, ran large batches as fast (plan: 4096 segments, 3.5e7
 // arguments, 408 us either way) but paid for up to 33 launches (plan-less: 480 us

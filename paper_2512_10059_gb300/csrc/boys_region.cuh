@@ -13,7 +13,7 @@
 //
 // What bounds it: the integer multiply pipe, which takes a 32 x 32 -> 64-bit
 // product every clock and SM (and also most moves and adds), at small K; the
-// stores at K = 32 (2^26 arguments of all regions: 2.69 ms, 1.00 of the measured
+// stores at K = 32 (2^26 arguments of all regions: 2.68 ms, 1.02 of the measured
 // copy bandwidth).  All terms of the downward step are positive: it never
 // cancels, one scaling per order serves every lane, and since every lane
 // produces the orders in the same sequence a warp stores whole rows as it goes
